@@ -329,23 +329,35 @@ MemberDesc make_desc(const shf_grid* o, const Member& m) {
   d.nyq_phi = m.nyq;
   d.nyq_omega = static_cast<char*>(m.nyq) + (size_t)m.ny * (o->precision == SHF_FP64 ? 8 : 4);
   d.st = m.d_st;
-  d.a = m.a; d.b = m.b; d.kappa = m.kappa; d.M = m.M; d.eta = m.eta; d.rho = m.rho;
-  d.gdot = m.gdot; d.dt = m.dt; d.dx = m.dx;
-  d.c_dt_aM = (m.dt * m.a) * m.M;
-  d.c_dt_bM = (m.dt * m.b) * m.M;
-  d.c_hdt_kM = 0.5 * ((m.dt * m.kappa) * m.M);
+  RealPar<double>& p = d.d;
+  p.a = m.a; p.b = m.b; p.kappa = m.kappa; p.dt = m.dt;
+  p.c_dt_aM = (m.dt * m.a) * m.M;
+  p.c_dt_bM = (m.dt * m.b) * m.M;
+  p.c_hdt_kM = 0.5 * ((m.dt * m.kappa) * m.M);
   d.stokes = m.rho == 0.0 ? 1 : 0;
-  d.c_hdt_nu = d.stokes ? 0.0 : 0.5 * (m.dt * (m.eta / m.rho));
-  d.c_force = d.stokes ? -1.0 / m.eta : -1.0 / m.rho;
-  d.inv_2h = 1.0 / (2.0 * m.dx);
-  d.inv_h2 = 1.0 / (m.dx * m.dx);
-  d.inv_4h2 = 1.0 / (4.0 * m.dx * m.dx);
-  d.inv_nxny = 1.0 / ((double)m.nx * (double)m.ny);
+  p.c_hdt_nu = d.stokes ? 0.0 : 0.5 * (m.dt * (m.eta / m.rho));
+  p.c_force = d.stokes ? -1.0 / m.eta : -1.0 / m.rho;
+  p.inv_2h = 1.0 / (2.0 * m.dx);
+  p.inv_h2 = 1.0 / (m.dx * m.dx);
+  p.inv_4h2 = 1.0 / (4.0 * m.dx * m.dx);
+  p.inv_nxny = 1.0 / ((double)m.nx * (double)m.ny);
   const double two_pi = 6.283185307179586476925286766559;
-  d.qx_unit = two_pi / (m.nx * m.dx);
-  d.qy_unit = two_pi / (m.ny * m.dx);
+  p.qx_unit = two_pi / (m.nx * m.dx);
+  p.qy_unit = two_pi / (m.ny * m.dx);
+  RealPar<float>& f = d.f;
+  f.a = (float)p.a; f.b = (float)p.b; f.kappa = (float)p.kappa; f.dt = (float)p.dt;
+  f.c_dt_aM = (float)p.c_dt_aM; f.c_dt_bM = (float)p.c_dt_bM; f.c_hdt_kM = (float)p.c_hdt_kM;
+  f.c_hdt_nu = (float)p.c_hdt_nu; f.c_force = (float)p.c_force;
+  f.inv_2h = (float)p.inv_2h; f.inv_h2 = (float)p.inv_h2; f.inv_4h2 = (float)p.inv_4h2;
+  f.inv_nxny = (float)p.inv_nxny; f.qx_unit = (float)p.qx_unit; f.qy_unit = (float)p.qy_unit;
+  d.qx_lo = (float)(p.qx_unit - (double)f.qx_unit);
+  const double fs = p.c_force * p.inv_2h * p.inv_2h;
+  d.force_scale.x = (float)fs;
+  d.force_scale.y = (float)(fs - (double)d.force_scale.x);
+  d.gdot_dt = m.gdot * m.dt;
   d.remap = o->remap_mode == SHF_REMAP_SHIFT ? 1 : 0;
   d.ratio = m.nx / m.ny;
+  d.inv_ratio = 1.0 / d.ratio;
   const bool fp32 = o->precision == SHF_FP32;
   d.w_hat = m.w_hat;
   d.low_rows = m.low_rows;
@@ -1261,7 +1273,9 @@ int shf_set_step(shf_grid* g, int64_t n) {
   if (g->kind == 2) return fail(g, SHF_EINVAL, "the step counter belongs to the ensemble");
   SHF_CUDA(g, cudaSetDevice(g->device));
   // the strain fields are recomputed on the device before the next step
-  std::vector<StepState> v(g->members.size(), StepState{(long long)n, 0, 0.0, 0.0});
+  StepState at{};
+  at.n = (long long)n;
+  std::vector<StepState> v(g->members.size(), at);
   SHF_CUDA(g, cudaMemcpyAsync(g->d_state, v.data(), v.size() * sizeof(StepState), cudaMemcpyHostToDevice,
                               g->stream));
   SHF_CUDA(g, cudaStreamSynchronize(g->stream));

@@ -15,6 +15,25 @@ struct StepState {
   long long n;
   long long dK;     // K(n+1) - K(n): nonzero when the strain wraps during the step
   double s0, s1;    // s(t^n), s(t^{n+1})
+  float2 f0, f1;    // s0 and s1 as float pairs (hi, lo): FP32 kernels convert nothing
+  float2 w0, w1;    // Eq. p1y's weights 1 - |s1|/2 and |s1|/2 as float pairs
+};
+
+// A member's parameters and derived constants in the working precision.  The
+// host rounds them once: a conversion or product in the kernels would go
+// through the FP64 pipe (1/64 of the FP32 rate, about 16 cycles of an SM per
+// warp instruction), and every thread of every launch used to make ten or more.
+template <class T>
+struct RealPar {
+  T a, b, kappa, dt;
+  T c_dt_aM;             // dt a M
+  T c_dt_bM;             // dt b M
+  T c_hdt_kM;            // dt kappa M / 2
+  T c_hdt_nu;            // dt (eta / rho) / 2      (inertial)
+  T c_force;             // -1/rho (inertial) or -1/eta (Stokes), multiplies F
+  T inv_2h, inv_h2, inv_4h2;
+  T inv_nxny;            // 1 / (nx ny), the inverse-transform normalisation
+  T qx_unit, qy_unit;    // 2 pi / (nx dx), 2 pi / (ny dx)
 };
 
 // Per-member descriptor, resident in device memory (one entry per run of a
@@ -52,16 +71,12 @@ struct MemberDesc {
   const void* tmap;
   int* err;       // device flag of the grid: a bounded wait in a kernel gave up (SHF_ETIMEOUT)
   StepState* st;  // device step counter and strain of the current step
-  // parameters and derived constants (double; cast to the working precision)
-  double a, b, kappa, M, eta, rho, gdot, dt, dx;
-  double c_dt_aM;        // dt a M
-  double c_dt_bM;        // dt b M
-  double c_hdt_kM;       // dt kappa M / 2
-  double c_hdt_nu;       // dt (eta / rho) / 2      (inertial)
-  double c_force;        // -1/rho (inertial) or -1/eta (Stokes), multiplies F
-  double inv_2h, inv_h2, inv_4h2;
-  double inv_nxny;       // 1 / (nx ny), the inverse-transform normalisation
-  double qx_unit, qy_unit;  // 2 pi / (nx dx), 2 pi / (ny dx)
+  double gdot_dt;        // gdot dt, the strain per step
+  double inv_ratio;      // 1 / ratio (exact: a power of two)
+  RealPar<double> d;     // parameters and derived constants
+  RealPar<float> f;      // the same, rounded
+  float qx_lo;           // qx_unit = f.qx_unit + qx_lo to about 2^-48
+  float2 force_scale;    // c_force inv_2h^2 as a float pair (k_lowrows_exact)
   int stokes;            // rho == 0
   int remap;             // 1 when the SHIFT remap is active
   int ratio;             // nx / ny
@@ -91,12 +106,12 @@ constexpr int kLowMExact = 8;
 // Strain sawtooth of Section V from the integer step n (same operation order
 // as the host and the oracle; explicit rounding intrinsics keep the compiler
 // from contracting it): total = (gdot dt) n, K = floor(total / r + 1/2),
-// s = total - K r.
-__device__ __forceinline__ void strain_dev(long long n, double gdot, double dt, int r, double& s,
+// s = total - K r.  r is a power of two, so the division is an exact product.
+__device__ __forceinline__ void strain_dev(long long n, double gdot_dt, double r, double inv_r, double& s,
                                            long long& K) {
-  const double total = __dmul_rn(__dmul_rn(gdot, dt), (double)n);
-  const double Kd = floor(__dadd_rn(__ddiv_rn(total, (double)r), 0.5));
-  s = __dsub_rn(total, __dmul_rn(Kd, (double)r));
+  const double total = __dmul_rn(gdot_dt, (double)n);
+  const double Kd = floor(__dadd_rn(__dmul_rn(total, inv_r), 0.5));
+  s = __dsub_rn(total, __dmul_rn(Kd, r));
   K = (long long)Kd;
 }
 

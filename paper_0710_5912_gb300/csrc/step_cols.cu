@@ -32,14 +32,39 @@ __device__ __forceinline__ void stage_column(cplx<T>* st, const cplx<T>* __restr
 template <class T>
 struct ColConsts {
   T norm, qyu, caM, cbM, ckM, cnu, dt;
-  double qx_unit, s_d;
+  T qxu, qxl, s, sl;                                   // qx_unit and s (FP32: hi and lo parts)
   int ny;
   bool stokes;
-  __device__ __forceinline__ ColConsts(const MemberDesc& D, int mode, int ny_)
-      : norm((T)D.inv_nxny), qyu((T)D.qy_unit), caM((T)D.c_dt_aM), cbM((T)D.c_dt_bM), ckM((T)D.c_hdt_kM),
-        cnu((T)D.c_hdt_nu), dt((T)D.dt), qx_unit(D.qx_unit),
-        s_d(mode == 0 ? D.st->s0 : D.st->s1),        // s^n for phi, s^{n+1} for flow
-        ny(ny_), stokes(D.stokes != 0) {}
+  __device__ __forceinline__ ColConsts(const MemberDesc& D, int mode, int ny_) : ny(ny_), stokes(D.stokes != 0) {
+    const RealPar<T>& p = par<T>(D);
+    norm = p.inv_nxny; qyu = p.qy_unit; caM = p.c_dt_aM; cbM = p.c_dt_bM; ckM = p.c_hdt_kM; cnu = p.c_hdt_nu;
+    dt = p.dt; qxu = p.qx_unit;
+    const StepState& S = *D.st;                         // s^n for phi, s^{n+1} for flow
+    if constexpr (sizeof(T) == 4) {
+      const float2 sp = mode == 0 ? S.f0 : S.f1;
+      qxl = D.qx_lo; s = sp.x; sl = sp.y;
+    } else {
+      qxl = T(0); s = mode == 0 ? S.s0 : S.s1; sl = T(0);
+    }
+  }
+  // qx = m qx_unit and s qx of mode m, each rounded once to the working
+  // precision: in FP32 both products are float pairs (errors by fused
+  // multiply-adds, about 2^-46), where forming them in double cost every
+  // thread four instructions on the FP64 pipe per item
+  __device__ __forceinline__ void mode_qx(int m, T& qx, T& sqx) const {
+    if constexpr (sizeof(T) == 4) {
+      const float mf = (float)m;
+      const float p = __fmul_rn(mf, qxu);
+      const float e = __fmaf_rn(mf, qxl, __fmaf_rn(mf, qxu, -p));
+      qx = __fadd_rn(p, e);
+      const float ql = __fadd_rn(__fsub_rn(p, qx), e);
+      const float h = __fmul_rn(s, qx);
+      sqx = __fadd_rn(h, __fmaf_rn(sl, qx, __fmaf_rn(s, ql, __fmaf_rn(s, qx, -h))));
+    } else {
+      qx = m * qxu;
+      sqx = s * qx;
+    }
+  }
 };
 
 // Quotients of the multipliers: FP32 takes the hardware reciprocal
@@ -52,7 +77,7 @@ __device__ __forceinline__ double quot(double a, double b) { return a / b; }
 // compile-time pass kind (0: phi; 1: inertial flow; 2: Stokes flow):
 // kind 0: va = phi*_hat -> increment of phi_hat (x norm), vb = f_hat;
 // kinds 1-2: va = g_hat -> psi_hat (x norm), vb = omega*_hat -> increment (x norm).
-// qx = m q_unit and sqx = s q_x, both formed in double.
+// qx and sqx = s q_x as ColConsts::mode_qx forms them.
 template <int KIND, class T>
 __device__ __forceinline__ void col_multiply_k(const ColConsts<T>& K, int m, T qx, T sqx, int nn, cplx<T>& va,
                                                cplx<T>& vb) {
@@ -198,9 +223,8 @@ __global__ void __launch_bounds__(512, min_ctas<T>()) k_colpass(const MemberDesc
     issue(m + stride);
     fft_reg<false>(va, log2ny, t, buf, tws);
     if (two) fft_reg<false>(vb, log2ny, t, buf, tws);
-    const double qx_d = mm * K.qx_unit;
-    const T qx = (T)qx_d;
-    const T sqx = (T)(K.s_d * qx_d);                    // s q_x formed in double
+    T qx, sqx;
+    K.mode_qx(mm, qx, sqx);
 #pragma unroll
     for (int q = 0; q < kP; ++q) col_multiply<T>(mode, K, mm, qx, sqx, t + q * Tc, va[q], vb[q]);
     fft_reg<true>(va, log2ny, t, buf, tws);
@@ -406,9 +430,8 @@ __device__ __forceinline__ void colpass_single_body(const MemberDesc& D, int log
 #pragma unroll
       for (int q = 0; q < P; ++q) low_override(D, mm, t + q * Tc, ny, a[q]);
     }
-    const double q_d = mm * K.qx_unit;
-    const T qx = (T)q_d;
-    const T sqx = (T)(K.s_d * q_d);                     // s q_x formed in double
+    T qx, sqx;
+    K.mode_qx(mm, qx, sqx);
     if (KIND == 1) {
       if (dK) {                                         // stage omega_hat^n so that rows can be relabelled
 #pragma unroll
@@ -555,9 +578,8 @@ __device__ __forceinline__ void colpass_chunk_body(const MemberDesc& D, int log2
 #pragma unroll
       for (int q = 0; q < P; ++q) low_override(D, mm, t + q * Tc, ny, a[q]);
     }
-    const double q_d = mm * K.qx_unit;
-    const T qx = (T)q_d;
-    const T sqx = (T)(K.s_d * q_d);                     // s q_x formed in double
+    T qx, sqx;
+    K.mode_qx(mm, qx, sqx);
     if (KIND == 1) {
       if (dK) {                                         // stage omega_hat^n so that rows can be relabelled
 #pragma unroll

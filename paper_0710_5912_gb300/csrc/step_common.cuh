@@ -14,12 +14,15 @@ template <class T> struct Layout;
 template <> struct Layout<float> { static constexpr int LC = 1; };   // 2 complex floats = 16 B
 template <> struct Layout<double> { static constexpr int LC = 0; };  // 1 complex double = 16 B
 
-// cells by which row j moves at a wrap: ((K1 - K0) r j) mod nx
+// cells by which row j moves at a wrap: ((K1 - K0) r j) mod nx (nx a power of two)
 __device__ __forceinline__ int remap_shift(long long dK, int r, int j, int nx) {
-  long long v = ((dK * r) % nx) * j % nx;
-  if (v < 0) v += nx;
-  return (int)v;
+  return (int)((unsigned long long)dK * (unsigned)r * (unsigned)j) & (nx - 1);
 }
+
+// the member's constants in the working precision
+template <class T> __device__ __forceinline__ const RealPar<T>& par(const MemberDesc& D);
+template <> __device__ __forceinline__ const RealPar<float>& par<float>(const MemberDesc& D) { return D.f; }
+template <> __device__ __forceinline__ const RealPar<double>& par<double>(const MemberDesc& D) { return D.d; }
 
 // x-spectral element (j, m) in the tiled layout
 __device__ __forceinline__ size_t xs_idx(int j, int m, int ny, int LC) {
@@ -36,7 +39,8 @@ struct Shear {
   long long dK;   // K(n+1) - K(n): nonzero when the strain wraps during the step
   // next = false: s = s(t^n) (stage 1); next = true: s = s(t^{n+1}) (stages 2-3)
   __device__ __forceinline__ Shear(const StepState& S, bool next) {
-    s = (T)(next ? S.s1 : S.s0);
+    if constexpr (sizeof(T) == 4) s = next ? S.f1.x : S.f0.x;
+    else s = next ? S.s1 : S.s0;
     w1 = (s < T(0) ? -s : s) * T(0.5);
     w0 = T(1) - w1;
     d = s >= T(0) ? -2 : 2;
@@ -45,16 +49,25 @@ struct Shear {
 };
 
 // one thread: the StepState of member D for the step starting at n
+__device__ __forceinline__ float2 float_pair(double v) {
+  const float h = (float)v;
+  return float2{h, (float)(v - (double)h)};
+}
 __device__ __forceinline__ void step_state_set(const MemberDesc& D, long long n) {
   double s0, s1;
   long long K0, K1;
-  strain_dev(n, D.gdot, D.dt, D.ratio, s0, K0);
-  strain_dev(n + 1, D.gdot, D.dt, D.ratio, s1, K1);
+  strain_dev(n, D.gdot_dt, (double)D.ratio, D.inv_ratio, s0, K0);
+  strain_dev(n + 1, D.gdot_dt, (double)D.ratio, D.inv_ratio, s1, K1);
+  const double w1 = 0.5 * (s1 < 0.0 ? -s1 : s1);
   StepState* S = D.st;
   S->n = n;
   S->dK = K1 - K0;
   S->s0 = s0;
   S->s1 = s1;
+  S->f0 = float_pair(s0);
+  S->f1 = float_pair(s1);
+  S->w0 = float_pair(1.0 - w1);
+  S->w1 = float_pair(w1);
 }
 
 
@@ -75,10 +88,6 @@ __device__ __forceinline__ float kahan_add(float s, float x, float& c) {
 struct F2 {
   float hi, lo;
 };
-__device__ __forceinline__ F2 f2_of(double v) {
-  const float h = (float)v;
-  return F2{h, (float)(v - (double)h)};
-}
 // Knuth's TwoSum: a + b = s + e exactly
 __device__ __forceinline__ F2 two_sum_f(float a, float b) {
   const float s = __fadd_rn(a, b);

@@ -139,10 +139,9 @@ __global__ void __launch_bounds__(kLxWarps * 32) k_lowrows_exact(const MemberDes
   __syncthreads();
   const Shear<float> sc(*D.st, true);                  // s^{n+1}
   {                                                    // mu in FP32, as the stage-2 stencil forms it
-    const float a = (float)D.a, b = (float)D.b, kappa = (float)D.kappa;
+    const float a = D.f.a, b = D.f.b, kappa = D.f.kappa;
     const float cxx = 1.f + sc.s * sc.s, cxy = 2.f * sc.s;
-    const float kxx = kappa * cxx * (float)D.inv_h2, kxy = kappa * cxy * (float)D.inv_4h2,
-                kyy = kappa * (float)D.inv_h2;
+    const float kxx = kappa * cxx * D.f.inv_h2, kxy = kappa * cxy * D.f.inv_4h2, kyy = kappa * D.f.inv_h2;
     for (int e = tid; e < 2 * (RT + 2) * (XT + 4); e += nt) {
       const int h = e / ((RT + 2) * (XT + 4)), e1 = e - h * (RT + 2) * (XT + 4);
       const int r = e1 / (XT + 4), c = e1 - r * (XT + 4);
@@ -156,10 +155,8 @@ __global__ void __launch_bounds__(kLxWarps * 32) k_lowrows_exact(const MemberDes
     }
   }
   __syncthreads();
-  const double s1 = D.st->s1;
-  const double w1d = 0.5 * (s1 < 0.0 ? -s1 : s1);
-  const F2 W0 = f2_of(1.0 - w1d), W1 = f2_of(w1d);
-  const F2 KF = f2_of(D.c_force * D.inv_2h * D.inv_2h);
+  const F2 W0{D.st->w0.x, D.st->w0.y}, W1{D.st->w1.x, D.st->w1.y};
+  const F2 KF{D.force_scale.x, D.force_scale.y};
   const int dd = sc.d;                                 // the diagonal's x offset at row j + 1
   const int lowm = D.lowm, nv = 2 * (lowm + 1);
   const int tshift = LOG2_NMAX - log2nx;

@@ -183,9 +183,10 @@ __device__ __forceinline__ void stage2_pair(const MemberDesc& D, const T* __rest
                                             int log2nx, int my, const Shear<T>& sc, int t, int Tf) {
   const int nx = 1 << log2nx, mx = nx - 1;
   const T cxx = T(1) + sc.s * sc.s, cxy = T(2) * sc.s;
-  const T kappa = (T)D.kappa;
-  const MuConsts<T> k{(T)D.a, (T)D.b, kappa * cxx * (T)D.inv_h2, kappa * cxy * (T)D.inv_4h2, kappa * (T)D.inv_h2};
-  const T inv2h = (T)D.inv_2h, cf = (T)D.c_force;
+  const RealPar<T>& par_ = par<T>(D);
+  const T kappa = par_.kappa;
+  const MuConsts<T> k{par_.a, par_.b, kappa * cxx * par_.inv_h2, kappa * cxy * par_.inv_4h2, kappa * par_.inv_h2};
+  const T inv2h = par_.inv_2h, cf = par_.c_force;
   auto row = [&](int j) { return phi + ((size_t)(j & my) << log2nx); };
   for (int q = t; q < (nx >> 2); q += Tf) {
     const int x0 = 4 * q;
@@ -421,7 +422,7 @@ __global__ void __launch_bounds__(rowfwd_cta_threads(P), rowfwd_min_ctas<T>(P))
   const T* psi = static_cast<const T*>(D.psi);
   const T* om = static_cast<const T*>(D.omega);
   const Shear<T> sc(*D.st, false);                     // s^n
-  const T dt = (T)D.dt, inv2h = (T)D.inv_2h;
+  const T dt = par<T>(D).dt, inv2h = par<T>(D).inv_2h;
   const bool inertial = !D.stokes;
   const bool wrap = D.remap && sc.dK != 0;
 
@@ -574,6 +575,10 @@ __global__ void __launch_bounds__(rowfwd_cta_threads(P), P == 16 ? 2 : min_ctas<
   }
   __syncthreads();
 
+  // the next step's state (no CTA of this launch reads it): its chain of FP64
+  // operations runs beside the first loads, not after the last store
+  if (mode == 1 && blockIdx.x == 0 && threadIdx.x == blockDim.x - 1) step_state_set(D, D.st->n + 1);
+
   auto issue = [&](int w) {
     if (w < nitems) {
       const int sub = w % nsub;
@@ -693,8 +698,6 @@ __global__ void __launch_bounds__(rowfwd_cta_threads(P), P == 16 ? 2 : min_ctas<
     }
   }
   cp_async_wait_all();
-  // the next step's state; no CTA of this launch reads it
-  if (mode == 1 && blockIdx.x == 0 && threadIdx.x == 0) step_state_set(D, D.st->n + 1);
 }
 
 // ----------------------------------------------------------------- launchers
