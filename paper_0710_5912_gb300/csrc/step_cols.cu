@@ -193,6 +193,7 @@ __global__ void __launch_bounds__(512, min_ctas<T>()) k_colpass(const MemberDesc
   C* in1 = static_cast<C*>(mode == 0 ? D.xs_f : D.xs_w);
   C* tws = reinterpret_cast<C*>(smem_raw + (size_t)ipc * colpass_inst_bytes(ny, sizeof(T)));
   stage_tables_to_smem(tws, tw, log2ny, kLogP, threadIdx.x, blockDim.x);
+  pdl_wait();
 
   auto issue = [&](int m) {
     if (m < nitems) {
@@ -278,6 +279,7 @@ template <int U>
 __global__ void __launch_bounds__(kLowColsWarps * 32) k_lowmode_cols(const MemberDesc* __restrict__ descs,
                                                                      int log2ny, const float4* __restrict__ twff) {
   const MemberDesc& D = descs[blockIdx.y];
+  pdl_wait();
   if (!D.low) return;                                  // uniform per CTA
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int o = blockIdx.x;
@@ -350,11 +352,11 @@ void launch_lowmode_cols(const MemberDesc* d, int nmem, int log2ny, const float4
   const int outs = (kLowM + 1) * (2 * kLowN + 1);
   const dim3 grid(outs, nmem);
   const int u = (1 << log2ny) / (kLowColsWarps * 32);
-  if (u >= 16) k_lowmode_cols<16><<<grid, kLowColsWarps * 32, 0, st>>>(d, log2ny, twff);
-  else if (u >= 8) k_lowmode_cols<8><<<grid, kLowColsWarps * 32, 0, st>>>(d, log2ny, twff);
-  else if (u >= 4) k_lowmode_cols<4><<<grid, kLowColsWarps * 32, 0, st>>>(d, log2ny, twff);
-  else if (u >= 2) k_lowmode_cols<2><<<grid, kLowColsWarps * 32, 0, st>>>(d, log2ny, twff);
-  else k_lowmode_cols<1><<<grid, kLowColsWarps * 32, 0, st>>>(d, log2ny, twff);
+  const void* f = u >= 16 ? (const void*)k_lowmode_cols<16> : u >= 8 ? (const void*)k_lowmode_cols<8>
+                : u >= 4  ? (const void*)k_lowmode_cols<4>  : u >= 2 ? (const void*)k_lowmode_cols<2>
+                          : (const void*)k_lowmode_cols<1>;
+  void* args[] = {(void*)&d, (void*)&log2ny, (void*)&twff};
+  launch_pdl(f, grid, kLowColsWarps * 32, args, 0, st);
 }
 
 // The FP32 column pass on single mode columns (ny < 512): item m = one mode,
@@ -385,9 +387,10 @@ __device__ __forceinline__ void colpass_single_body(const MemberDesc& D, int log
   C* in1 = static_cast<C*>(KIND == 0 ? D.xs_f : D.xs_w);
   C* what = static_cast<C*>(D.w_hat);
   // a wrap during the step relabels omega_hat^n: (m, n) <- (m, n + m dK)
-  const int dK = (KIND == 1 && D.remap) ? (int)(D.st->dK & (ny - 1)) : 0;
   C* tws = reinterpret_cast<C*>(smem_raw + (size_t)ipc * colsingle_inst_bytes(ny));
   stage_tables_to_smem(tws, tw, log2ny, 4, threadIdx.x, blockDim.x);
+  pdl_wait();
+  const int dK = (KIND == 1 && D.remap) ? (int)(D.st->dK & (ny - 1)) : 0;
 
   auto issue = [&](int m) {
     if (m < nitems) {
@@ -498,7 +501,6 @@ __device__ __forceinline__ void colpass_chunk_body(const MemberDesc& D, int log2
   C* in0 = static_cast<C*>(KIND == 0 ? D.xs_phi : (KIND == 4 ? D.xs_w : D.xs_g));
   C* in1 = static_cast<C*>(KIND == 0 ? D.xs_f : D.xs_w);
   C* what = static_cast<C*>(D.w_hat);
-  const int dK = (KIND == 1 && D.remap) ? (int)(D.st->dK & (ny - 1)) : 0;
   C* tws = reinterpret_cast<C*>(smem_raw + colchunk_cta_bytes(ny));
   stage_tables_to_smem(tws, tw, log2ny, 4, threadIdx.x, blockDim.x);
 
@@ -526,6 +528,8 @@ __device__ __forceinline__ void colpass_chunk_body(const MemberDesc& D, int log2
     mbar_init_fence();
   }
   __syncthreads();
+  pdl_wait();
+  const int dK = (KIND == 1 && D.remap) ? (int)(D.st->dK & (ny - 1)) : 0;
   auto issue = [&](int cb) {
     if (cb < nitems && threadIdx.x == 0) {
       fence_proxy_async_smem();                         // the stage's earlier reads come first
@@ -664,9 +668,11 @@ void launch_col_kernel(int kind, const MemberDesc* d, int nmem, int log2nx, int 
       const MemberDesc* dd = d;
       const float2* tt = tw;
       void* args[] = {(void*)&dd, (void*)&log2nx, (void*)&tt};
-      cudaLaunchKernel(colpass_fp32_fn<LN>(k), grid, dim3(c.threads), args, c.smem, st);
-    } else
-      k_colpass<T, LN><<<grid, c.threads, c.smem, st>>>(d, log2nx, tw, mode);
+      launch_pdl(colpass_fp32_fn<LN>(k), grid, c.threads, args, c.smem, st);
+    } else {
+      void* args[] = {(void*)&d, (void*)&log2nx, (void*)&tw, (void*)&mode};
+      launch_pdl((const void*)k_colpass<T, LN>, grid, c.threads, args, c.smem, st);
+    }
   });
 }
 

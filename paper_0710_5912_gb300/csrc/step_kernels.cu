@@ -119,6 +119,7 @@ __device__ __forceinline__ void df_acc_prod(F2& acc, F2 F, float wh, float wl) {
 __global__ void __launch_bounds__(kLxWarps * 32) k_lowrows_exact(const MemberDesc* __restrict__ descs, int log2nx,
                                                                  int log2ny, const float4* __restrict__ twff) {
   const MemberDesc& D = descs[blockIdx.z];
+  pdl_wait();
   if (D.low != 2) return;                              // uniform per CTA
   extern __shared__ __align__(16) float sm[];
   const int nx = 1 << log2nx, ny = 1 << log2ny, mx = nx - 1, my = ny - 1;
@@ -250,7 +251,8 @@ void launch_lowrows_exact(const MemberDesc* d, int nmem, int log2nx, int log2ny,
   const int nx = 1 << log2nx, ny = 1 << log2ny;
   const size_t smem = (size_t)lowexact_smem_floats(nx, ny) * sizeof(float);
   const dim3 grid((nx / 2) / lowexact_cols(nx), ny / lowexact_rows(ny), nmem);
-  k_lowrows_exact<<<grid, kLxWarps * 32, smem, st>>>(d, log2nx, log2ny, twff);
+  void* args[] = {(void*)&d, (void*)&log2nx, (void*)&log2ny, (void*)&twff};
+  launch_pdl((const void*)k_lowrows_exact, grid, kLxWarps * 32, args, smem, st);
 }
 size_t lowrows_bytes(int nx, int ny) {
   // hi and lo planes of the coefficients, the exact path's per-tile sums and

@@ -248,6 +248,7 @@ __global__ void __launch_bounds__(rowfwd_cta_threads(P), rowfwd_min_ctas<T>(P)) 
   const T* src = mode == 1 ? static_cast<const T*>(D.phi) : static_cast<const T*>(D.omega);
   C* tws = reinterpret_cast<C*>(smem_raw + (size_t)ipc * rowfwd_inst_bytes(nx, sizeof(T)));
   stage_tables_to_smem(tws, tw, log2nx, log2_points<P>(), threadIdx.x, blockDim.x);
+  pdl_wait();
   const Shear<T> sc(*D.st, true);                      // stage 2: s^{n+1}
   const int my = ny - 1;
 
@@ -418,6 +419,7 @@ __global__ void __launch_bounds__(rowfwd_cta_threads(P), rowfwd_min_ctas<T>(P))
   T* bufw = reinterpret_cast<T*>(smem_raw + (size_t)inst * 2 * one + one);
   C* tws = reinterpret_cast<C*>(smem_raw + (size_t)ipc * 2 * one);
   stage_tables_to_smem(tws, tw, log2nx, log2_points<P>(), threadIdx.x, blockDim.x);
+  pdl_wait();
   const T* phi = static_cast<const T*>(D.phi);
   const T* psi = static_cast<const T*>(D.psi);
   const T* om = static_cast<const T*>(D.omega);
@@ -574,6 +576,7 @@ __global__ void __launch_bounds__(rowfwd_cta_threads(P), P == 16 ? 2 : min_ctas<
     for (int k = 0; k < 3; ++k) tmap_acquire(tmaps + 128 * k);
   }
   __syncthreads();
+  pdl_wait();
 
   // the next step's state (no CTA of this launch reads it): its chain of FP64
   // operations runs beside the first loads, not after the last store
@@ -737,7 +740,7 @@ void launch_row_kernel(int kind, const MemberDesc* d, int nmem, int log2nx, int 
       const MemberDesc* dd = d;
       const cplx<T>* tt = tw;
       void* args[] = {(void*)&dd, (void*)&log2ny, (void*)&tt};
-      cudaLaunchKernel(stage1_fn<T, LN>(c.variant), grid, dim3(c.threads), args, c.smem, st);
+      launch_pdl(stage1_fn<T, LN>(c.variant), grid, c.threads, args, c.smem, st);
     });
     return;
   }
@@ -750,7 +753,7 @@ void launch_row_kernel(int kind, const MemberDesc* d, int nmem, int log2nx, int 
     const MemberDesc* dd = d;
     const cplx<T>* tt = tw;
     void* args[] = {(void*)&dd, (void*)&log2ny, (void*)&tt};
-    cudaLaunchKernel(f, grid, dim3(c.threads), args, c.smem, st);
+    launch_pdl(f, grid, c.threads, args, c.smem, st);
   });
 }
 
