@@ -234,6 +234,12 @@ LaunchCfg persistent_cfg(int kind, int nfft, int max_inst, int items, size_t ins
   if (ipc < 1) ipc = 1;
   if (ipc > max_inst) ipc = max_inst;
   while (ipc > 1 && ipc * inst_bytes + tab + extra > kSmemLimit) ipc /= 2;
+  // small grids: whole warps spread over the chip rather than full CTAs on a
+  // few SMs (packed, 128 row pairs of 256 points made 8 CTAs): until the launch
+  // has two CTAs per SM.  A CTA's instances share nothing but its barriers and
+  // its copy of the twiddle table.  Per step: 256^2 FP32 49.3 -> 40.6 us, 64^2
+  // FP64 257 -> 125 us, 512^2 FP64 807 -> 231 us (the FP64 pipe is per SM)
+  while (ipc > 1 && ipc * Tf > 32 && (long long)(items / ipc) * nmem < 2 * sm_count()) ipc /= 2;
   c.inst_per_cta = ipc;
   c.threads = ipc * Tf;
   c.smem = ipc * inst_bytes + tab + extra;
