@@ -330,6 +330,11 @@ struct NamedSync {
     asm volatile("bar.sync %0, %1;\n" ::"r"(id), "r"(nthreads) : "memory");
   }
 };
+// a group's barrier where a kernel runs as thread groups, else the CTA's
+template <bool GROUPED> struct GroupSync : NamedSync {};
+template <> struct GroupSync<false> : CtaSync {
+  __device__ __forceinline__ GroupSync(NamedSync) {}
+};
 
 template <bool INV, int LR, bool LAST, int P, class C, class Sync = CtaSync>
 __device__ __forceinline__ void fft_reg_stage(C (&v)[P], int log2N, int log2Ns, int t, C* buf, const C* twt,
@@ -391,12 +396,12 @@ __device__ __forceinline__ void fft_reg(C (&v)[P], int log2N, int t, C* buf, con
 }
 
 // v[q] = X[t + T q] -> buf (padded, natural order), followed by a barrier.
-template <int P, class C>
-__device__ __forceinline__ void reg_to_smem(const C (&v)[P], int log2N, int t, C* buf) {
+template <int P, class C, class Sync = CtaSync>
+__device__ __forceinline__ void reg_to_smem(const C (&v)[P], int log2N, int t, C* buf, const Sync& sync = Sync{}) {
   const int T = 1 << (log2N - log2_points<P>());
 #pragma unroll
   for (int q = 0; q < P; ++q) buf[pad16(t + q * T)] = v[q];
-  __syncthreads();
+  sync();
 }
 
 }  // namespace shf

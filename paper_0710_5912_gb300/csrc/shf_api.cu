@@ -221,8 +221,9 @@ int sm_count() {
 // query), shared over the members of the launch.
 template <class T>
 LaunchCfg persistent_cfg(int kind, int nfft, int max_inst, int items, size_t inst_bytes, int nmem, int P = kP,
-                         size_t extra = 0) {
+                         size_t extra = 0, int groups = 1) {
   LaunchCfg c{};
+  c.groups = groups;
   const bool fwd = kind == KIND_STAGE1 || kind == KIND_STAGE2;
   const bool rows = fwd || kind == KIND_ROWINV_PHI || kind == KIND_ROWINV_FLOW;
   const int cta = (rows || P == 16) ? rowfwd_cta_threads(P) : 512;   // FP32 column passes: 16 points, 256 threads
@@ -233,6 +234,7 @@ LaunchCfg persistent_cfg(int kind, int nfft, int max_inst, int items, size_t ins
   int ipc = cta / Tf;
   if (ipc < 1) ipc = 1;
   if (ipc > max_inst) ipc = max_inst;
+  while (ipc > 1 && groups * ipc * Tf > (P == 16 ? 768 : 512)) ipc /= 2;
   while (ipc > 1 && ipc * inst_bytes + tab + extra > kSmemLimit) ipc /= 2;
   // small grids: whole warps spread over the chip rather than full CTAs on a
   // few SMs (packed, 128 row pairs of 256 points made 8 CTAs): until the launch
@@ -245,12 +247,29 @@ LaunchCfg persistent_cfg(int kind, int nfft, int max_inst, int items, size_t ins
   c.smem = ipc * inst_bytes + tab + extra;
   c.variant = rows ? P : 0;
   const int work = (items + ipc - 1) / ipc;
-  const int resident = step_kernel_occupancy<T>(kind, log2n, c.variant, c.threads, c.smem) * sm_count();
+  const int resident = step_kernel_occupancy<T>(kind, log2n, c.variant, c.threads, groups, c.smem) * sm_count();
   int g = (resident + nmem - 1) / nmem;
   if (g > work) g = work;
   c.grid_x = g < 1 ? 1 : g;
   c.grid_y = 1;
   return c;
+}
+
+// Thread groups per CTA of the forward row passes (stage 1: up to three, one
+// per transform of an item; stage 2: two, the transform and the low row
+// modes).  One group's transforms follow one another in the item's threads,
+// which keeps a full chip busy; where the row pairs of a launch are too few for
+// that, the groups run them side by side and share the stencil: as long as all
+// pairs' groups fit on the chip at once (768 threads per SM at 80 registers;
+// FP64: 512), and a group is whole warps.
+template <class T>
+int stage_groups(int want, int nx, int ny, int nmem, int P) {
+  const int Tf = nx / P, per_sm = P == 16 ? 768 : 512;
+  if (P == 8 && sizeof(T) == 4) return 1;
+  if (Tf * (ny / 2) < 32) return 1;
+  int g = want;
+  while (g > 1 && ((long long)g * Tf * (ny / 2) * nmem > (long long)per_sm * sm_count() || g * Tf > per_sm)) --g;
+  return g;
 }
 
 // The tuning knobs of a size class: points per thread of the fused stage-1
@@ -274,10 +293,13 @@ void configure_class_t(SizeClass& cl, Tune tune) {
   tune = resolved<T>(cl, tune);
   const size_t R = sizeof(T), Cx = 2 * R;
   const int nx = cl.nx, ny = cl.ny, nmem = (int)cl.members.size();
-  cl.cfg[KIND_STAGE1] = persistent_cfg<T>(KIND_STAGE1, nx, ny / 2, ny / 2, 2 * stage1_inst_bytes(nx, R), nmem,
-                                           tune.stage1_points);
-  cl.cfg[KIND_STAGE2] = persistent_cfg<T>(KIND_STAGE2, nx, ny / 2, ny / 2, rowfwd_inst_bytes(nx, R), nmem,
-                                           tune.stage2_points);
+  // (a pair of groups only would leave inertial members a transform behind)
+  const int g1 = stage_groups<T>(3, nx, ny, nmem, tune.stage1_points) == 3 ? 3 : 1;
+  const int g2 = stage_groups<T>(2, nx, ny, nmem, tune.stage2_points);
+  cl.cfg[KIND_STAGE1] = persistent_cfg<T>(KIND_STAGE1, nx, ny / 2, ny / 2, (g1 > 1 ? 3 : 2) * stage1_inst_bytes(nx, R), nmem,
+                                           tune.stage1_points, 0, g1);
+  cl.cfg[KIND_STAGE2] = persistent_cfg<T>(KIND_STAGE2, nx, ny / 2, ny / 2, rowfwd_inst_bytes(nx, R, g2), nmem,
+                                           tune.stage2_points, 0, g2);
   // column items: single mode columns with 16 points per thread (FP32), or
   // whole 16-byte chunks of one complex double with 8 (FP64)
   const int ncol_items = nx / 2;
@@ -290,7 +312,7 @@ void configure_class_t(SizeClass& cl, Tune tune) {
     c.inst_per_cta = 1;
     c.threads = 2 * (ny / 16);
     c.smem = colchunk_cta_bytes(ny) + stage_table_bytes(cl.log2ny, 4, R) + kColBarBytes;
-    const int resident = step_kernel_occupancy<T>(KIND_COLPASS_PHI, cl.log2ny, 0, c.threads, c.smem) * sm_count();
+    const int resident = step_kernel_occupancy<T>(KIND_COLPASS_PHI, cl.log2ny, 0, c.threads, 1, c.smem) * sm_count();
     int g = (resident + nmem - 1) / nmem;
     if (g > nx / 4) g = nx / 4;
     c.grid_x = g < 1 ? 1 : g;
@@ -653,6 +675,11 @@ void launch_kind(shf_grid* o, SizeClass& cl, int kind, cudaStream_t st) {
     return;
   }
   LaunchCfg c = cl.cfg[kind];
+  if (kind == KIND_STAGE1 && c.groups == 3) {           // Stokes members have two transforms
+    bool inertial = false;
+    for (int r : cl.members) inertial = inertial || o->members[r].rho > 0.0;
+    if (!inertial) c.groups = 2;
+  }
   if (kind == KIND_COLPASS_FLOW) {                      // the flow pass specialised on the members' regime
     bool inertial = false, stokes = false;
     for (int r : cl.members) (o->members[r].rho > 0.0 ? inertial : stokes) = true;

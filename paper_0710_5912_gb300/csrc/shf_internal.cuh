@@ -121,8 +121,9 @@ __device__ __forceinline__ void strain_dev(long long n, double gdot_dt, double r
 // one x-spectral chunk column of each input field plus the buffer; rowinv
 // stages the 32-byte chunks of a row pair (nx complex) plus the buffer.
 __host__ __device__ constexpr size_t round128(size_t b) { return (b + 127) & ~(size_t)127; }
-__host__ __device__ constexpr size_t rowfwd_inst_bytes(int nx, size_t real_bytes) {
-  return round128(2 * (size_t)nx * real_bytes + (size_t)padded_len(nx) * 2 * real_bytes);
+// (with several groups a second buffer for the low modes' terms)
+__host__ __device__ constexpr size_t rowfwd_inst_bytes(int nx, size_t real_bytes, int groups) {
+  return round128(2 * (size_t)nx * real_bytes + (groups > 1 ? 2 : 1) * (size_t)padded_len(nx) * 2 * real_bytes);
 }
 // the FP64 column pass stages two columns of 16-byte complex doubles plus
 // the padded exchange buffer
@@ -167,7 +168,13 @@ __host__ __device__ constexpr size_t stage_table_bytes(int log2n, int LP, size_t
 // yields the force's low modes) and the FP32 inverse rows P = 16 (8% faster
 // than 8 in the flow pass, equal in the phi pass at 4096^2).
 constexpr int rowfwd_cta_threads(int P) { return P == 16 ? 256 : 512; }
-template <class T> constexpr int rowfwd_min_ctas(int P) { return P == 16 ? 3 : (sizeof(T) == 4 ? 2 : 1); }
+// launch bounds of the forward row passes: with P = 16 three CTAs of one group
+// or up to three groups of 256 threads in one CTA (stage_groups); with P = 8
+// the groups share the 512 threads
+template <class T> constexpr int rows_max_threads(int P, bool grouped) { return P == 16 ? (grouped ? 768 : 256) : 512; }
+template <class T> constexpr int rows_min_ctas(int P, bool grouped) {
+  return P == 16 ? (grouped ? 1 : 3) : (sizeof(T) == 4 ? 2 : 1);
+}
 template <class T> constexpr int rowfwd_default_points() { return sizeof(T) == 4 ? 16 : 8; }
 template <class T> constexpr int rowinv_default_points() { return sizeof(T) == 4 ? 16 : 8; }
 
@@ -188,7 +195,8 @@ enum { KIND_ROWFWD_OMEGA = 100, KIND_COLPASS_WINIT = 101 };
 
 struct LaunchCfg {
   int grid_x, grid_y;   // grid (the member index is the last grid dimension)
-  int threads;
+  int threads;          // of one group
+  int groups;           // thread groups per CTA (blockDim.y), see stage_groups
   size_t smem;          // dynamic shared memory bytes
   int inst_per_cta;     // transform instances per CTA (persistent kinds)
   int variant;          // rows: points per thread (8, 16);
@@ -197,13 +205,13 @@ struct LaunchCfg {
 
 template <class T> void launch_step_kernel(int kind, const MemberDesc* d, int nmem, int log2nx, int log2ny,
                                            const cplx<T>* tw, const LaunchCfg& c, cudaStream_t st);
-template <class T> int step_kernel_occupancy(int kind, int log2n, int variant, int threads, size_t smem);
+template <class T> int step_kernel_occupancy(int kind, int log2n, int variant, int threads, int groups, size_t smem);
 // the transform kernels by family (step_rows.cu, step_cols.cu)
 template <class T> void launch_row_kernel(int kind, const MemberDesc* d, int nmem, int log2nx, int log2ny,
                                           const cplx<T>* tw, const LaunchCfg& c, cudaStream_t st);
 template <class T> void launch_col_kernel(int kind, const MemberDesc* d, int nmem, int log2nx, int log2ny,
                                           const cplx<T>* tw, const LaunchCfg& c, cudaStream_t st);
-template <class T> int row_kernel_occupancy(int kind, int log2nx, int variant, int threads, size_t smem);
+template <class T> int row_kernel_occupancy(int kind, int log2nx, int variant, int threads, int groups, size_t smem);
 template <class T> int col_kernel_occupancy(int log2ny, int threads, size_t smem);
 template <class T> void set_row_smem_limits(int lim);
 template <class T> void set_col_smem_limits(int lim);

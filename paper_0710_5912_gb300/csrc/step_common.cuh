@@ -265,13 +265,13 @@ __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wai
 // cost more than the overlap gave (1024^2: 89 us after the wait, 94 at the start).
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
 // launch of a kernel that calls pdl_wait
-inline void launch_pdl(const void* f, dim3 grid, int threads, void** args, size_t smem, cudaStream_t st) {
+inline void launch_pdl(const void* f, dim3 grid, dim3 threads, void** args, size_t smem, cudaStream_t st) {
   cudaLaunchAttribute at{};
   at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at.val.programmaticStreamSerializationAllowed = 1;
   cudaLaunchConfig_t c{};
   c.gridDim = grid;
-  c.blockDim = dim3(threads);
+  c.blockDim = threads;
   c.dynamicSmemBytes = smem;
   c.stream = st;
   c.attrs = &at;

@@ -278,9 +278,9 @@ void launch_step_kernel(int kind, const MemberDesc* d, int nmem, int log2nx, int
 // CTAs of a persistent kind that fit on one SM at (threads, smem); log2n is the
 // kind's transform length (log2 nx for row kinds, log2 ny for column kinds)
 template <class T>
-int step_kernel_occupancy(int kind, int log2n, int variant, int threads, size_t smem) {
+int step_kernel_occupancy(int kind, int log2n, int variant, int threads, int groups, size_t smem) {
   if (kind == KIND_COLPASS_PHI || kind == KIND_COLPASS_FLOW) return col_kernel_occupancy<T>(log2n, threads, smem);
-  return row_kernel_occupancy<T>(kind, log2n, variant, threads, smem);
+  return row_kernel_occupancy<T>(kind, log2n, variant, threads, groups, smem);
 }
 
 template <class T>
@@ -294,7 +294,7 @@ void set_step_smem_limits() {
 #define SHF_INST(T)                                                                                      \
   template void launch_step_kernel<T>(int, const MemberDesc*, int, int, int, const cplx<T>*,             \
                                       const LaunchCfg&, cudaStream_t);                                    \
-  template int step_kernel_occupancy<T>(int, int, int, int, size_t);                                      \
+  template int step_kernel_occupancy<T>(int, int, int, int, int, size_t);                                      \
   template void set_step_smem_limits<T>();
 
 SHF_INST(float)

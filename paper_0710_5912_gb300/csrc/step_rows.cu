@@ -74,10 +74,10 @@ __device__ __forceinline__ void low_row_terms(const float* stage, float* Zb, con
 }
 
 // Part 2, after a barrier: the compensated sums and the rows' coefficients.
-// All threads of the CTA call it (barriers).
-template <int LN>
-__device__ __forceinline__ void low_row_reduce(float* Zb, int t, const MemberDesc& D, int p, bool active,
-                                               int log2ny) {
+// All threads of the group that `sync` joins call it.
+template <int LN, class Sync>
+__device__ __forceinline__ void low_row_reduce(float* Zb, int t, const MemberDesc& D, int p, bool active, int log2ny,
+                                               const Sync& sync) {
   const int lowm = D.lowm;
   const int nv = 2 * (2 * lowm + 1);                   // real values per thread
   constexpr int Tc = (1 << LN) / 16;                   // threads per instance
@@ -93,12 +93,12 @@ __device__ __forceinline__ void low_row_reduce(float* Zb, int t, const MemberDes
       const int t0 = gi * per, t1 = min(Tc, t0 + per);
       for (int tt = t0; tt < t1; ++tt) s = kahan_add(s, Zb[k * Tc + tt], c);
     }
-    __syncthreads();
+    sync();
     if (has) {
       Zb[2 * t] = s;
       Zb[2 * t + 1] = c;
     }
-    __syncthreads();
+    sync();
   }
   // level 2: value k = t + i Tc folds its G partials (or its Tc terms) in order
   float tot[kSlots];
@@ -118,11 +118,11 @@ __device__ __forceinline__ void low_row_reduce(float* Zb, int t, const MemberDes
     }
     tot[i] = __fsub_rn(s, c);                          // Kahan's c is the excess added
   }
-  __syncthreads();
+  sync();
 #pragma unroll
   for (int i = 0; i < kSlots; ++i)
     if (t + i * Tc < nv) Zb[t + i * Tc] = tot[i];
-  __syncthreads();
+  sync();
   for (int m = t; active && m <= lowm; m += Tc) {     // short rows have fewer threads than modes
     const float zr = Zb[2 * m], zi = Zb[2 * m + 1];
     const float nr = m ? Zb[2 * (lowm + m)] : zr, ni = m ? Zb[2 * (lowm + m) + 1] : zi;
@@ -130,7 +130,7 @@ __device__ __forceinline__ void low_row_reduce(float* Zb, int t, const MemberDes
     lr[2 * p] = float2{0.5f * (zr + nr), 0.5f * (zi - ni)};
     lr[2 * p + 1] = float2{0.5f * (zi + ni), -0.5f * (zr - nr)};
   }
-  __syncthreads();
+  sync();
 }
 
 // ===================================================== stage-2 stencil of a row pair
@@ -227,8 +227,11 @@ __device__ __forceinline__ void stage2_pair(const MemberDesc& D, const T* __rest
 // memory and transforms a + i b, so every output chunk of the pair is one
 // whole 32-byte piece.  (Stage 1's row transforms are fused with its
 // stencil: k_stage1_rows.)
-template <class T, int LN, int P, int MODE>
-__global__ void __launch_bounds__(rowfwd_cta_threads(P), rowfwd_min_ctas<T>(P)) k_rowfwd(const MemberDesc* __restrict__ descs, int log2ny,
+// Mode 1 runs as G = blockDim.y groups of threads (see stage_groups): all
+// groups share the stencil; then group 0 transforms while group 1 forms the
+// low row modes in a buffer of its own.
+template <class T, int LN, int P, int MODE, bool GROUPED = false>
+__global__ void __launch_bounds__(rows_max_threads<T>(P, GROUPED), rows_min_ctas<T>(P, GROUPED)) k_rowfwd(const MemberDesc* __restrict__ descs, int log2ny,
                                                                const cplx<T>* __restrict__ tw) {
   constexpr int mode = MODE;
   constexpr int log2nx = LN;
@@ -240,14 +243,19 @@ __global__ void __launch_bounds__(rowfwd_cta_threads(P), rowfwd_min_ctas<T>(P)) 
   const int Tf = nx / P;
   const int ipc = blockDim.x / Tf;
   const int inst = threadIdx.x / Tf, t = threadIdx.x - inst * Tf;
+  const int G = GROUPED ? blockDim.y : 1, grp = GROUPED ? threadIdx.y : 0;
+  const GroupSync<GROUPED> sync{NamedSync{1 + grp, (int)blockDim.x}};
   const int nitems = mode == 2 && !D.wspec ? 0 : ny >> 1;
   const int stride = gridDim.x * ipc;
-  unsigned char* base = smem_raw + (size_t)inst * rowfwd_inst_bytes(nx, sizeof(T));
+  const size_t inst_bytes = rowfwd_inst_bytes(nx, sizeof(T), G);
+  unsigned char* base = smem_raw + (size_t)inst * inst_bytes;
   T* stage = reinterpret_cast<T*>(base);
   C* Z = reinterpret_cast<C*>(base + 2 * (size_t)nx * sizeof(T));
+  C* Zlow = G > 1 ? Z + padded_len(nx) : Z;            // group 1's buffer for the low modes' terms
+  const int lowgrp = G > 1 ? 1 : 0;
   const T* src = mode == 1 ? static_cast<const T*>(D.phi) : static_cast<const T*>(D.omega);
-  C* tws = reinterpret_cast<C*>(smem_raw + (size_t)ipc * rowfwd_inst_bytes(nx, sizeof(T)));
-  stage_tables_to_smem(tws, tw, log2nx, log2_points<P>(), threadIdx.x, blockDim.x);
+  C* tws = reinterpret_cast<C*>(smem_raw + (size_t)ipc * inst_bytes);
+  stage_tables_to_smem(tws, tw, log2nx, log2_points<P>(), grp * blockDim.x + threadIdx.x, G * blockDim.x);
   pdl_wait();
   const Shear<T> sc(*D.st, true);                      // stage 2: s^{n+1}
   const int my = ny - 1;
@@ -261,7 +269,7 @@ __global__ void __launch_bounds__(rowfwd_cta_threads(P), rowfwd_min_ctas<T>(P)) 
     cp_async_commit();
   };
   auto prefetch = [&](int w) {                         // mode 1: ask L2 for phi's rows 2w - 2 .. 2w + 3
-    if (w < nitems && t < 6) l2_prefetch(src + ((size_t)((2 * w - 2 + t) & my) << log2nx), (unsigned)(nx * sizeof(T)));
+    if (w < nitems && grp == 0 && t < 6) l2_prefetch(src + ((size_t)((2 * w - 2 + t) & my) << log2nx), (unsigned)(nx * sizeof(T)));
   };
 
   const int iters = persistent_iters(nitems, ipc);
@@ -273,8 +281,8 @@ __global__ void __launch_bounds__(rowfwd_cta_threads(P), rowfwd_min_ctas<T>(P)) 
     const int p = w;
     if constexpr (MODE == 1) {
       const int j0 = 2 * (active ? w : 0);
-      if (sc.d > 0) stage2_pair<true>(D, src, stage, j0, log2nx, my, sc, t, Tf);
-      else stage2_pair<false>(D, src, stage, j0, log2nx, my, sc, t, Tf);
+      if (sc.d > 0) stage2_pair<true>(D, src, stage, j0, log2nx, my, sc, grp * Tf + t, G * Tf);
+      else stage2_pair<false>(D, src, stage, j0, log2nx, my, sc, grp * Tf + t, G * Tf);
       __syncthreads();                                 // the pair's g complete
       prefetch(w + stride);                            // the next item's rows, during the transform
     } else {
@@ -282,23 +290,28 @@ __global__ void __launch_bounds__(rowfwd_cta_threads(P), rowfwd_min_ctas<T>(P)) 
       __syncthreads();
     }
     if constexpr (sizeof(T) == 4 && P == 16 && MODE == 1) {   // the force's low row modes, part 1
-      if (D.low == 1) low_row_terms<LN>(reinterpret_cast<const float*>(stage), reinterpret_cast<float*>(Z), tws, t, D);
+      if (D.low == 1 && grp == lowgrp)
+        low_row_terms<LN>(reinterpret_cast<const float*>(stage), reinterpret_cast<float*>(Zlow), tws, t, D);
     }
     C v[P];
+    if (grp == 0) {
 #pragma unroll
-    for (int q = 0; q < P; ++q) {
-      const int i = t + q * Tf;
-      v[q] = C{stage[i], stage[nx + i]};
+      for (int q = 0; q < P; ++q) {
+        const int i = t + q * Tf;
+        v[q] = C{stage[i], stage[nx + i]};
+      }
     }
     __syncthreads();                                    // stage free
     if (MODE == 2) issue(w + stride);                   // next item streams in during the transform
     if constexpr (sizeof(T) == 4 && P == 16 && MODE == 1) {
-      if (D.low == 1) low_row_reduce<LN>(reinterpret_cast<float*>(Z), t, D, p, active, log2ny);
+      if (D.low == 1 && grp == lowgrp) low_row_reduce<LN>(reinterpret_cast<float*>(Zlow), t, D, p, active, log2ny, sync);
     }
-    fft_reg<false>(v, log2nx, t, Z, tws);
-    reg_to_smem(v, log2nx, t, Z);
-    if (active) write_pair_rows<LC>(Z, static_cast<C*>(mode == 1 ? D.xs_g : D.xs_w), 2 * p, nx, ny, t, Tf);
-    __syncthreads();                                    // Z reads done before the next transform
+    if (grp == 0) {
+      fft_reg<false>(v, log2nx, t, Z, tws, sync);
+      reg_to_smem(v, log2nx, t, Z, sync);
+      if (active) write_pair_rows<LC>(Z, static_cast<C*>(mode == 1 ? D.xs_g : D.xs_w), 2 * p, nx, ny, t, Tf);
+      sync();                                           // Z reads done before the next transform
+    }
   }
   cp_async_wait_all();
 }
@@ -399,8 +412,11 @@ __device__ __forceinline__ void stage1_pair(const T* phi, const T* psi, const T*
   }
 }
 
-template <class T, int LN, int P>
-__global__ void __launch_bounds__(rowfwd_cta_threads(P), rowfwd_min_ctas<T>(P))
+// With G = blockDim.y > 1 groups of threads (stage_groups) the item's stencil
+// is shared by all groups and each of its transforms is one group's, side by
+// side on buffers of their own; with one group they follow one another.
+template <class T, int LN, int P, bool GROUPED>
+__global__ void __launch_bounds__(rows_max_threads<T>(P, GROUPED), rows_min_ctas<T>(P, GROUPED))
     k_stage1_rows(const MemberDesc* __restrict__ descs, int log2ny, const cplx<T>* __restrict__ tw) {
   constexpr int log2nx = LN;
   using C = cplx<T>;
@@ -413,12 +429,18 @@ __global__ void __launch_bounds__(rowfwd_cta_threads(P), rowfwd_min_ctas<T>(P))
   const int inst = threadIdx.x / Tf, t = threadIdx.x - inst * Tf;
   const int nitems = ny >> 1;
   const int stride = gridDim.x * ipc;
-  // two padded buffers per instance: phi*'s pair, then omega*'s (or a's)
+  const int G = GROUPED ? blockDim.y : 1, grp = GROUPED ? threadIdx.y : 0;
+  const GroupSync<GROUPED> sync{NamedSync{1 + grp, (int)blockDim.x}};
+  // two padded buffers per instance: phi*'s pair, then omega*'s (or a's); f is
+  // transformed in phi*'s when that is done, or with several groups in a third
+  // one (Stokes members of two groups: the second)
+  const int nbuf = G > 2 ? 3 : 2;
   const size_t one = stage1_inst_bytes(nx, sizeof(T));
-  T* bufp = reinterpret_cast<T*>(smem_raw + (size_t)inst * 2 * one);
-  T* bufw = reinterpret_cast<T*>(smem_raw + (size_t)inst * 2 * one + one);
-  C* tws = reinterpret_cast<C*>(smem_raw + (size_t)ipc * 2 * one);
-  stage_tables_to_smem(tws, tw, log2nx, log2_points<P>(), threadIdx.x, blockDim.x);
+  T* bufp = reinterpret_cast<T*>(smem_raw + (size_t)inst * nbuf * one);
+  T* bufw = reinterpret_cast<T*>(smem_raw + (size_t)inst * nbuf * one + one);
+  T* buff = G == 1 ? bufp : reinterpret_cast<T*>(smem_raw + (size_t)inst * nbuf * one + (nbuf - 1) * one);
+  C* tws = reinterpret_cast<C*>(smem_raw + (size_t)ipc * nbuf * one);
+  stage_tables_to_smem(tws, tw, log2nx, log2_points<P>(), grp * blockDim.x + threadIdx.x, G * blockDim.x);
   pdl_wait();
   const T* phi = static_cast<const T*>(D.phi);
   const T* psi = static_cast<const T*>(D.psi);
@@ -430,7 +452,7 @@ __global__ void __launch_bounds__(rowfwd_cta_threads(P), rowfwd_min_ctas<T>(P))
 
   // ask L2 for item w's input rows (j0 - 1 .. j1 + 1 of phi, psi, omega)
   auto prefetch = [&](int w) {
-    if (w < nitems && t < 4) {
+    if (w < nitems && grp == 0 && t < 4) {
       const int j = (2 * w - 1 + t) & my;
       const unsigned bytes = (unsigned)nx * sizeof(T);
       l2_prefetch(phi + ((size_t)j << log2nx), bytes);
@@ -448,10 +470,10 @@ __global__ void __launch_bounds__(rowfwd_cta_threads(P), rowfwd_min_ctas<T>(P))
       const int i = t + q * Tf;
       v[q] = C{buf[i], buf[nx + i]};
     }
-    __syncthreads();                                   // buf becomes the exchange buffer
+    sync();                                            // buf becomes the exchange buffer
     C* Z = reinterpret_cast<C*>(buf);
-    fft_reg<false>(v, log2nx, t, Z, tws);
-    reg_to_smem(v, log2nx, t, Z);
+    fft_reg<false>(v, log2nx, t, Z, tws, sync);
+    reg_to_smem(v, log2nx, t, Z, sync);
     if (active) {
       write_pair_rows<LC>(Z, dst, 2 * p, nx, ny, t, Tf);
       if (nyq && t == 0) {
@@ -460,8 +482,9 @@ __global__ void __launch_bounds__(rowfwd_cta_threads(P), rowfwd_min_ctas<T>(P))
         nyq[2 * p + 1] = zn.y;
       }
     }
-    __syncthreads();                                   // Z read before buf is written again
+    sync();                                            // Z read before buf is written again
   };
+  const int ts = grp * Tf + t, Ts = G * Tf;            // this thread's place in the stencil
 
   const int iters = persistent_iters(nitems, ipc);
   int w = blockIdx.x * ipc + inst;
@@ -476,21 +499,21 @@ __global__ void __launch_bounds__(rowfwd_cta_threads(P), rowfwd_min_ctas<T>(P))
       const int sh1 = wrap ? remap_shift(sc.dK, D.ratio, j0 + 1, nx) : 0;
       T* gom = (active && !D.wspec) ? static_cast<T*>(D.omega_star) : (T*)nullptr;
       if (D.wspec) {
-        if (sc.d > 0) stage1_pair<true, true, true>(phi, psi, om, bufp, bufw, gphi, gom, j0, log2nx, my, sc, dt, inv2h, t, Tf, sh0, sh1);
-        else stage1_pair<false, true, true>(phi, psi, om, bufp, bufw, gphi, gom, j0, log2nx, my, sc, dt, inv2h, t, Tf, sh0, sh1);
+        if (sc.d > 0) stage1_pair<true, true, true>(phi, psi, om, bufp, bufw, gphi, gom, j0, log2nx, my, sc, dt, inv2h, ts, Ts, sh0, sh1);
+        else stage1_pair<false, true, true>(phi, psi, om, bufp, bufw, gphi, gom, j0, log2nx, my, sc, dt, inv2h, ts, Ts, sh0, sh1);
       } else {
-        if (sc.d > 0) stage1_pair<true, false, true>(phi, psi, om, bufp, bufw, gphi, gom, j0, log2nx, my, sc, dt, inv2h, t, Tf, sh0, sh1);
-        else stage1_pair<false, false, true>(phi, psi, om, bufp, bufw, gphi, gom, j0, log2nx, my, sc, dt, inv2h, t, Tf, sh0, sh1);
+        if (sc.d > 0) stage1_pair<true, false, true>(phi, psi, om, bufp, bufw, gphi, gom, j0, log2nx, my, sc, dt, inv2h, ts, Ts, sh0, sh1);
+        else stage1_pair<false, false, true>(phi, psi, om, bufp, bufw, gphi, gom, j0, log2nx, my, sc, dt, inv2h, ts, Ts, sh0, sh1);
       }
     } else {
-      if (sc.d > 0) stage1_pair<true, false, false>(phi, psi, om, bufp, bufw, gphi, (T*)nullptr, j0, log2nx, my, sc, dt, inv2h, t, Tf, 0, 0);
-      else stage1_pair<false, false, false>(phi, psi, om, bufp, bufw, gphi, (T*)nullptr, j0, log2nx, my, sc, dt, inv2h, t, Tf, 0, 0);
+      if (sc.d > 0) stage1_pair<true, false, false>(phi, psi, om, bufp, bufw, gphi, (T*)nullptr, j0, log2nx, my, sc, dt, inv2h, ts, Ts, 0, 0);
+      else stage1_pair<false, false, false>(phi, psi, om, bufp, bufw, gphi, (T*)nullptr, j0, log2nx, my, sc, dt, inv2h, ts, Ts, 0, 0);
     }
     __syncthreads();                                   // both staged pairs complete
     prefetch(w + stride);                              // the next item's rows, during the transforms
-    transform_pair(bufp, active, static_cast<C*>(D.xs_phi), static_cast<T*>(D.nyq_phi), p);
+    if (grp == 0) transform_pair(bufp, active, static_cast<C*>(D.xs_phi), static_cast<T*>(D.nyq_phi), p);
     // f = phi^3 of the pre-advection pair, in the FFT's register layout (the rows are in L1/L2)
-    {
+    if (G == 1 || grp == 1) {
       C v[P];
       const T* ra = phi + ((size_t)j0 << log2nx);
       const T* rb = ra + nx;
@@ -500,14 +523,15 @@ __global__ void __launch_bounds__(rowfwd_cta_threads(P), rowfwd_min_ctas<T>(P))
         const T a = ra[i], b = rb[i];
         v[q] = C{(a * a) * a, (b * b) * b};
       }
-      C* Z = reinterpret_cast<C*>(bufp);
-      fft_reg<false>(v, log2nx, t, Z, tws);
-      reg_to_smem(v, log2nx, t, Z);
+      C* Z = reinterpret_cast<C*>(buff);
+      fft_reg<false>(v, log2nx, t, Z, tws, sync);
+      reg_to_smem(v, log2nx, t, Z, sync);
       if (active) write_pair_rows<LC>(Z, static_cast<C*>(D.xs_f), j0, nx, ny, t, Tf);
-      __syncthreads();
+      sync();
     }
-    if (inertial)
+    if (inertial && (G == 1 || grp == 2))
       transform_pair(bufw, active, static_cast<C*>(D.xs_w), D.wspec ? (T*)nullptr : static_cast<T*>(D.nyq_omega), p);
+    if (G > 1) __syncthreads();                        // every group's buffer may be written again
   }
 }
 
@@ -704,30 +728,27 @@ __global__ void __launch_bounds__(rowfwd_cta_threads(P), P == 16 ? 2 : min_ctas<
 }
 
 // ----------------------------------------------------------------- launchers
-// the row kernels by variant P (points per thread; FP64 has P = 8 only) and
-// mode (0: phi, 1: g or flow), each compiled separately
-// the forward row kernels by P and mode (1: g, 2: omega into xs_w)
+// the forward row kernels by mode (1: g, 2: omega into xs_w) and thread groups
 template <class T, int LN>
-const void* rowfwd_fn(int P, int mode) {
-  if constexpr (sizeof(T) == 4) {
-    if (P == 16) return mode == 1 ? (const void*)k_rowfwd<T, LN, 16, 1> : (const void*)k_rowfwd<T, LN, 16, 2>;
-  }
-  return mode == 1 ? (const void*)k_rowfwd<T, LN, 8, 1> : (const void*)k_rowfwd<T, LN, 8, 2>;
+const void* rowfwd_fn(int mode, bool grouped) {
+  constexpr int P = rowfwd_default_points<T>();
+  if (mode == 2) return (const void*)k_rowfwd<T, LN, P, 2>;
+  return grouped ? (const void*)k_rowfwd<T, LN, P, 1, true> : (const void*)k_rowfwd<T, LN, P, 1, false>;
 }
 template <class T, int LN>
-const void* rowinv_fn(int P, int mode) {
-  if constexpr (sizeof(T) == 4) {
-    if (P == 16) return mode == 0 ? (const void*)k_rowinv<T, LN, 16, 0> : (const void*)k_rowinv<T, LN, 16, 1>;
-  }
-  return mode == 0 ? (const void*)k_rowinv<T, LN, 8, 0> : (const void*)k_rowinv<T, LN, 8, 1>;
+const void* rowinv_fn(int mode) {
+  constexpr int P = rowinv_default_points<T>();
+  return mode == 0 ? (const void*)k_rowinv<T, LN, P, 0> : (const void*)k_rowinv<T, LN, P, 1>;
 }
 
 template <class T, int LN>
-const void* stage1_fn(int P) {
+const void* stage1_fn(int P, bool grouped) {
   if constexpr (sizeof(T) == 4) {
-    if (P == 16) return (const void*)k_stage1_rows<T, LN, 16>;
+    if (P == 16) return grouped ? (const void*)k_stage1_rows<T, LN, 16, true> : (const void*)k_stage1_rows<T, LN, 16, false>;
+    return (const void*)k_stage1_rows<T, LN, 8, false>;
+  } else {
+    return grouped ? (const void*)k_stage1_rows<T, LN, 8, true> : (const void*)k_stage1_rows<T, LN, 8, false>;
   }
-  return (const void*)k_stage1_rows<T, LN, 8>;
 }
 
 template <class T>
@@ -740,7 +761,7 @@ void launch_row_kernel(int kind, const MemberDesc* d, int nmem, int log2nx, int 
       const MemberDesc* dd = d;
       const cplx<T>* tt = tw;
       void* args[] = {(void*)&dd, (void*)&log2ny, (void*)&tt};
-      launch_pdl(stage1_fn<T, LN>(c.variant), grid, c.threads, args, c.smem, st);
+      launch_pdl(stage1_fn<T, LN>(c.variant, c.groups > 1), grid, dim3(c.threads, c.groups), args, c.smem, st);
     });
     return;
   }
@@ -749,21 +770,21 @@ void launch_row_kernel(int kind, const MemberDesc* d, int nmem, int log2nx, int 
   const int mode = fwd ? (kind == KIND_ROWFWD_OMEGA ? 2 : 1) : (kind == KIND_ROWINV_PHI ? 0 : 1);
   with_log2n(log2nx, [&](auto L) {
     constexpr int LN = decltype(L)::value;
-    const void* f = fwd ? rowfwd_fn<T, LN>(c.variant, mode) : rowinv_fn<T, LN>(c.variant, mode);
+    const void* f = fwd ? rowfwd_fn<T, LN>(mode, c.groups > 1) : rowinv_fn<T, LN>(mode);
     const MemberDesc* dd = d;
     const cplx<T>* tt = tw;
     void* args[] = {(void*)&dd, (void*)&log2ny, (void*)&tt};
-    launch_pdl(f, grid, c.threads, args, c.smem, st);
+    launch_pdl(f, grid, dim3(c.threads, kind == KIND_STAGE2 ? c.groups : 1), args, c.smem, st);
   });
 }
 
 template <class T>
-int row_kernel_occupancy(int kind, int log2nx, int variant, int threads, size_t smem) {
+int row_kernel_occupancy(int kind, int log2nx, int variant, int threads, int groups, size_t smem) {
   int nb = 0;
   if (kind == KIND_STAGE1) {
     with_log2n(log2nx, [&](auto L) {
       constexpr int LN = decltype(L)::value;
-      if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, stage1_fn<T, LN>(variant), threads, smem) != cudaSuccess)
+      if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, stage1_fn<T, LN>(variant, groups > 1), threads * groups, smem) != cudaSuccess)
         nb = 1;
     });
     return nb < 1 ? 1 : nb;
@@ -772,8 +793,8 @@ int row_kernel_occupancy(int kind, int log2nx, int variant, int threads, size_t 
   const int mode = fwd ? 1 : (kind == KIND_ROWINV_PHI ? 0 : 1);
   with_log2n(log2nx, [&](auto L) {
     constexpr int LN = decltype(L)::value;
-    const void* f = fwd ? rowfwd_fn<T, LN>(variant, mode) : rowinv_fn<T, LN>(variant, mode);
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, f, threads, smem) != cudaSuccess) nb = 1;
+    const void* f = fwd ? rowfwd_fn<T, LN>(mode, groups > 1) : rowinv_fn<T, LN>(mode);
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, f, threads * groups, smem) != cudaSuccess) nb = 1;
   });
   return nb < 1 ? 1 : nb;
 }
@@ -783,25 +804,26 @@ void set_row_smem_limits(int lim) {
   for (int ln = 4; ln <= LOG2_NMAX; ++ln)
     with_log2n(ln, [&](auto L) {
       constexpr int LN = decltype(L)::value;
-      for (int P : {8, 16})
-        cudaFuncSetAttribute(stage1_fn<T, LN>(P), cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-      for (int P : {8, 16})
-        for (int mode : {0, 1, 2}) {
-          if (mode > 0)
-            cudaFuncSetAttribute(rowfwd_fn<T, LN>(P, mode), cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-          if (mode < 2)
-            cudaFuncSetAttribute(rowinv_fn<T, LN>(P, mode), cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-        }
+      auto set = [&](const void* f) { cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, lim); };
+      for (bool grouped : {false, true}) {
+        for (int P : {8, 16}) set(stage1_fn<T, LN>(P, grouped));
+        for (int mode : {1, 2}) set(rowfwd_fn<T, LN>(mode, grouped));
+      }
+      for (int mode : {0, 1}) set(rowinv_fn<T, LN>(mode));
     });
 }
 
 #define SHF_ROW_INST(T)                                                                                   \
   template void launch_row_kernel<T>(int, const MemberDesc*, int, int, int, const cplx<T>*, const LaunchCfg&, \
                                      cudaStream_t);                                                        \
-  template int row_kernel_occupancy<T>(int, int, int, int, size_t);                                        \
+  template int row_kernel_occupancy<T>(int, int, int, int, int, size_t);                                        \
   template void set_row_smem_limits<T>(int);
 
-SHF_ROW_INST(float)
+// one translation unit per precision (step_rows_f64.cu includes this file)
+#ifdef SHF_ROWS_F64
 SHF_ROW_INST(double)
+#else
+SHF_ROW_INST(float)
+#endif
 
 }  // namespace shf
