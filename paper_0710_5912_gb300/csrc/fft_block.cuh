@@ -91,50 +91,6 @@ __device__ __forceinline__ void dft8(C* v) {
   v[7] = csub(e3, t3);
 }
 
-// radix 16 as 4 x 4: radix-4 DFTs over n1 (n = 4 n1 + n2), the factors
-// w16^{n2 k1}, w16 = exp(sigma 2 pi i / 16), then radix-4 DFTs over n2;
-// X[k1 + 4 k2] lands in v[k1 + 4 k2]
-template <bool INV, class C>
-__device__ __forceinline__ C w16_times(C x, int e) {
-  using T = decltype(x.x);
-  const T c1 = T(0.92387953251128675612818318939678828682), s1 = T(0.38268343236508977172845998403039886676);
-  const T r2 = T(0.70710678118654752440084436210484903928);
-  const T sg = INV ? T(1) : T(-1);                     // sign of the imaginary part of w16
-  T cr, ci;                                            // w16^e = cr + i sg ci
-  switch (e) {
-    case 1: cr = c1; ci = s1; break;
-    case 2: cr = r2; ci = r2; break;
-    case 3: cr = s1; ci = c1; break;
-    case 4: return mul_si<INV>(x);
-    case 6: cr = -r2; ci = r2; break;
-    case 9: cr = -c1; ci = -s1; break;
-    default: return x;
-  }
-  const T wi = sg * ci;
-  return C{x.x * cr - x.y * wi, x.x * wi + x.y * cr};
-}
-template <bool INV, class C>
-__device__ __forceinline__ void dft16(C* v) {
-#pragma unroll
-  for (int n2 = 0; n2 < 4; ++n2) dft4<INV>(v[n2], v[4 + n2], v[8 + n2], v[12 + n2]);   // -> v[4 k1 + n2]
-#pragma unroll
-  for (int n2 = 1; n2 < 4; ++n2)
-#pragma unroll
-    for (int k1 = 1; k1 < 4; ++k1) v[4 * k1 + n2] = w16_times<INV>(v[4 * k1 + n2], n2 * k1);
-  C o[16];
-#pragma unroll
-  for (int k1 = 0; k1 < 4; ++k1) {
-    C a = v[4 * k1], b = v[4 * k1 + 1], c = v[4 * k1 + 2], d = v[4 * k1 + 3];
-    dft4<INV>(a, b, c, d);
-    o[k1] = a;
-    o[k1 + 4] = b;
-    o[k1 + 8] = c;
-    o[k1 + 12] = d;
-  }
-#pragma unroll
-  for (int q = 0; q < 16; ++q) v[q] = o[q];
-}
-
 template <bool INV, class C>
 __device__ __forceinline__ C twiddle(const C* __restrict__ tw, int idx) {
   C w = __ldg(tw + idx);
@@ -238,8 +194,7 @@ __host__ __device__ constexpr int padded_len(int N) { return N + N / 16; }
 // (exp(+2 pi i k / L), exp(+2 pi i 2k / L)) for k = 0..Ns-1 at entries
 // [2 (stage_table_offset(a, LR) + k)], [.. + 1]: one 16-byte load (FP32) per
 // butterfly, and the warp's loads are one contiguous run.  The other factors
-// are products of these two (at most two roundings deep): w3 = w1 w2,
-// w4 = w2 w2, w5 = w4 w1, w6 = w4 w2, w7 = w4 w3.
+// are products of these two (stage_factors, dit_twiddled).
 __host__ __device__ constexpr int stage_table_offset(int a, int LR) {
   return 4 * ((1 << a) - 1) + (LR - 1) * (1 << a);
 }
@@ -281,12 +236,66 @@ __device__ __forceinline__ void load_pair(const double2* p, double2& w1, double2
   w2 = p[1];
 }
 
-// the R factors W_L^{k r}, r = 0..R-1, of butterfly k of a stage, from the
-// compact table of a transform with 2^LP points per thread
-template <int R, int LP, class C>
-__device__ __forceinline__ void load_stage_factors(const C* tab, int log2Ns, int k, C (&f)[R]) {
-  C w1, w2;
-  load_pair(tab + 2 * (compact_stage_offset(log2Ns, LP) + k), w1, w2);
+// ---- the arithmetic of the register FFT.  Products whose contraction would
+// depend on their surroundings are spelled out, so that kernels that share a
+// formula give the same bits.
+__device__ __forceinline__ float fma_rn(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double fma_rn(double a, double b, double c) { return __fma_rn(a, b, c); }
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+template <class C> __device__ __forceinline__ C cmul_rn(C a, C b) {
+  return C{fma_rn(a.x, b.x, -mul_rn(a.y, b.y)), fma_rn(a.x, b.y, mul_rn(a.y, b.x))};
+}
+template <class C> __device__ __forceinline__ C csqr_rn(C a) {
+  return C{fma_rn(a.x, a.x, -mul_rn(a.y, a.y)), mul_rn(a.x + a.x, a.y)};
+}
+
+// -- FP32: radix-R DFTs of additions, the inputs multiplied by W^r first.
+// radix 16 as 4 x 4: radix-4 DFTs over n1 (n = 4 n1 + n2), the factors
+// w16^{n2 k1}, w16 = exp(sigma 2 pi i / 16), then radix-4 DFTs over n2;
+// X[k1 + 4 k2] lands in v[k1 + 4 k2]
+template <bool INV>
+__device__ __forceinline__ float2 w16_times(float2 x, int e) {
+  const float c1 = 0.92387953251128675612818318939678828682f, s1 = 0.38268343236508977172845998403039886676f;
+  const float r2 = 0.70710678118654752440084436210484903928f;
+  const float sg = INV ? 1.f : -1.f;                   // sign of the imaginary part of w16
+  float cr, ci;                                        // w16^e = cr + i sg ci
+  switch (e) {
+    case 1: cr = c1; ci = s1; break;
+    case 2: cr = r2; ci = r2; break;
+    case 3: cr = s1; ci = c1; break;
+    case 4: return mul_si<INV>(x);
+    case 6: cr = -r2; ci = r2; break;
+    case 9: cr = -c1; ci = -s1; break;
+    default: return x;
+  }
+  const float wi = sg * ci;
+  return float2{x.x * cr - x.y * wi, x.x * wi + x.y * cr};
+}
+template <bool INV>
+__device__ __forceinline__ void dft16(float2* v) {
+#pragma unroll
+  for (int n2 = 0; n2 < 4; ++n2) dft4<INV>(v[n2], v[4 + n2], v[8 + n2], v[12 + n2]);   // -> v[4 k1 + n2]
+#pragma unroll
+  for (int n2 = 1; n2 < 4; ++n2)
+#pragma unroll
+    for (int k1 = 1; k1 < 4; ++k1) v[4 * k1 + n2] = w16_times<INV>(v[4 * k1 + n2], n2 * k1);
+  float2 o[16];
+#pragma unroll
+  for (int k1 = 0; k1 < 4; ++k1) {
+    float2 a = v[4 * k1], b = v[4 * k1 + 1], c = v[4 * k1 + 2], d = v[4 * k1 + 3];
+    dft4<INV>(a, b, c, d);
+    o[k1] = a;
+    o[k1 + 4] = b;
+    o[k1 + 8] = c;
+    o[k1 + 12] = d;
+  }
+#pragma unroll
+  for (int q = 0; q < 16; ++q) v[q] = o[q];
+}
+// the R factors W^r, r = 1..R-1, from W and W^2 (at most three roundings deep)
+template <int R>
+__device__ __forceinline__ void stage_factors(float2 w1, float2 w2, float2 (&f)[R]) {
   f[1] = w1;
   if (R > 2) {
     f[2] = w2;
@@ -304,13 +313,105 @@ __device__ __forceinline__ void load_stage_factors(const C* tab, int log2Ns, int
     for (int r = 1; r < 8; ++r) f[8 + r] = cmul(f[8], f[r]);
   }
 }
-
-template <bool INV, int LR, class C>
-__device__ __forceinline__ void dft_radix(C* v) {
+template <bool INV, int LR>
+__device__ __forceinline__ void dft_radix(float2* v) {
   if (LR == 4) dft16<INV>(v);
   else if (LR == 3) dft8<INV>(v);
   else if (LR == 2) dft4<INV>(v[0], v[1], v[2], v[3]);
   else dft2<INV>(v[0], v[1]);
+}
+
+// -- FP64: X[k] = sum_r x_r W^r w_R^{r k} by decimation in time: with E, O the
+// transforms of the even and odd inputs (factor W^2),
+//   X[k] = E[k] + (W w_R^k) O[k],  X[k + R/2] = E[k] - (W w_R^k) O[k],
+// so a level of length len has the factors W^{R/len} w_len^k, and each
+// two-point butterfly takes its factor in six fused multiply-adds: four for
+// a + w b and one per component for a - w b = 2a - (a + w b).  10 FP64
+// instructions per point of a radix-8 stage, where separate factors (R - 1
+// products and their powers) and additions took 13; these passes are bound by
+// the FP64 pipe (about 16 cycles of an SM per warp instruction): a 1024^2 step
+// went from 916 to 796 us.  In FP32 the same butterflies gained 3% at 4096^2
+// and nothing below, and re-drew the rounding noise of phi; it keeps the form
+// above.
+// (a, b) <- (a + w b, a - w b)
+template <class C> __device__ __forceinline__ void bfly(C& a, C& b, C w) {
+  using T = decltype(a.x);
+  const C p = C{fma_rn(w.x, b.x, fma_rn(-w.y, b.y, a.x)), fma_rn(w.x, b.y, fma_rn(w.y, b.x, a.y))};
+  b = C{fma_rn(T(2), a.x, -p.x), fma_rn(T(2), a.y, -p.y)};
+  a = p;
+}
+// the same for w = sigma i (a quarter turn) times the given factor: (a, b) <- (a + i s w b, a - i s w b)
+template <bool INV, class C> __device__ __forceinline__ void bfly_quarter(C& a, C& b, C w) { bfly(a, b, mul_si<INV>(w)); }
+// w = 1, w = sigma i, and w = (1 + sigma i) / sqrt(2) turned by Q quarters
+template <class C> __device__ __forceinline__ void bfly_one(C& a, C& b) { dft2<false>(a, b); }
+template <bool INV, int Q, class C> __device__ __forceinline__ void bfly_eighth(C& a, C& b) {
+  using T = decltype(a.x);
+  const T c = T(0.70710678118654752440084436210484904);
+  const T sg = INV ? T(1) : T(-1);
+  // (1 + sg i) b, for Q = 1 sg i (1 + sg i) b = (-1 + sg i) b
+  const C d = Q == 0 ? C{b.x - sg * b.y, b.y + sg * b.x} : C{-b.x - sg * b.y, sg * b.x - b.y};
+  b = C{fma_rn(-c, d.x, a.x), fma_rn(-c, d.y, a.y)};
+  a = C{fma_rn(c, d.x, a.x), fma_rn(c, d.y, a.y)};
+}
+template <int LR> __host__ __device__ constexpr int bit_reversed(int r) {
+  int v = 0;
+  for (int i = 0; i < LR; ++i) v |= ((r >> i) & 1) << (LR - 1 - i);
+  return v;
+}
+constexpr double kCos8 = 0.70710678118654752440084436210484903928;
+// y holds the R inputs in bit-reversed places, factors all one; X in natural order
+template <bool INV, int LR, class C>
+__device__ __forceinline__ void dit_plain(C* y) {
+  using T = decltype(y[0].x);
+  constexpr int R = 1 << LR;
+  const T sg = INV ? T(1) : T(-1);
+#pragma unroll
+  for (int i = 0; i < R; i += 2) bfly_one(y[i], y[i + 1]);
+  if (LR >= 2)
+#pragma unroll
+    for (int i = 0; i < R; i += 4) {
+      bfly_one(y[i], y[i + 2]);
+      y[i + 3] = mul_si<INV>(y[i + 3]);
+      bfly_one(y[i + 1], y[i + 3]);
+    }
+  if (LR >= 3)
+#pragma unroll
+    for (int i = 0; i < R; i += 8) {
+      bfly_one(y[i], y[i + 4]);
+      bfly_eighth<INV, 0>(y[i + 1], y[i + 5]);
+      y[i + 6] = mul_si<INV>(y[i + 6]);
+      bfly_one(y[i + 2], y[i + 6]);
+      bfly_eighth<INV, 1>(y[i + 3], y[i + 7]);
+    }
+}
+// the same with the factors W^r, w1 = W and w2 = W^2 given (already of the transform's sign)
+template <bool INV, int LR, class C>
+__device__ __forceinline__ void dit_twiddled(C* y, C w1, C w2) {
+  using T = decltype(y[0].x);
+  constexpr int R = 1 << LR;
+  const T sg = INV ? T(1) : T(-1);
+  const C w4 = LR >= 3 ? csqr_rn(w2) : w2;
+  const C e8 = C{T(kCos8), sg * T(kCos8)};
+#pragma unroll
+  for (int i = 0; i < R; i += 2) bfly(y[i], y[i + 1], LR == 3 ? w4 : LR == 2 ? w2 : w1);
+  if (LR >= 2) {
+    const C w = LR == 3 ? w2 : w1;
+#pragma unroll
+    for (int i = 0; i < R; i += 4) {
+      bfly(y[i], y[i + 2], w);
+      bfly_quarter<INV>(y[i + 1], y[i + 3], w);
+    }
+  }
+  if (LR >= 3) {
+    const C we = cmul_rn(w1, e8);
+#pragma unroll
+    for (int i = 0; i < R; i += 8) {
+      bfly(y[i], y[i + 4], w1);
+      bfly(y[i + 1], y[i + 5], we);
+      bfly_quarter<INV>(y[i + 2], y[i + 6], w1);
+      bfly_quarter<INV>(y[i + 3], y[i + 7], we);
+    }
+  }
 }
 
 // One stage on the register layout.  LAST: keep the outputs in registers;
@@ -349,14 +450,21 @@ __device__ __forceinline__ void fft_reg_stage(C (&v)[P], int log2N, int log2Ns, 
     const int j = t + b * T;
     const int k = j & (Ns - 1);
 #pragma unroll
-    for (int r = 0; r < R; ++r) w[r] = v[b + r * B];
-    if (log2Ns > 0) {
-      C f[R];
-      load_stage_factors<R, log2_points<P>()>(twt, log2Ns, k, f);
+    for (int r = 0; r < R; ++r) w[sizeof(w[0].x) == 4 ? r : bit_reversed<LR>(r)] = v[b + r * B];
+    C w1, w2;
+    if (log2Ns > 0) load_pair(twt + 2 * (compact_stage_offset(log2Ns, log2_points<P>()) + k), w1, w2);
+    if constexpr (sizeof(w[0].x) == 4) {
+      if (log2Ns > 0) {
+        C f[R];
+        stage_factors<R>(w1, w2, f);
 #pragma unroll
-      for (int r = 1; r < R; ++r) w[r] = cmul(w[r], INV ? f[r] : cconj(f[r]));
+        for (int r = 1; r < R; ++r) w[r] = cmul(w[r], INV ? f[r] : cconj(f[r]));
+      }
+      dft_radix<INV, LR>(w);
+    } else {
+      if (log2Ns > 0) dit_twiddled<INV, LR>(w, INV ? w1 : cconj(w1), INV ? w2 : cconj(w2));
+      else dit_plain<INV, LR>(w);
     }
-    dft_radix<INV, LR>(w);
     if (LAST) {
 #pragma unroll
       for (int r = 0; r < R; ++r) v[b + r * B] = w[r];

@@ -319,6 +319,8 @@ void configure_class_t(SizeClass& cl, Tune tune) {
     c.grid_y = 1;
     cl.cfg[KIND_COLPASS_PHI] = c;
   }
+  LaunchCfg grouped{};
+  if (R == 8 && colgroup_cfg(nx, ny, nmem, sm_count(), &grouped)) cl.cfg[KIND_COLPASS_PHI] = grouped;
   cl.cfg[KIND_COLPASS_FLOW] = cl.cfg[KIND_COLPASS_PHI];
   const int PI = rowinv_default_points<T>();
   cl.cfg[KIND_ROWINV_PHI] = persistent_cfg<T>(KIND_ROWINV_PHI, nx, ny / 2, ny / 2, rowinv_inst_bytes(nx, R), nmem, PI,

@@ -213,6 +213,8 @@ template <class T> void launch_col_kernel(int kind, const MemberDesc* d, int nme
                                           const cplx<T>* tw, const LaunchCfg& c, cudaStream_t st);
 template <class T> int row_kernel_occupancy(int kind, int log2nx, int variant, int threads, int groups, size_t smem);
 template <class T> int col_kernel_occupancy(int log2ny, int threads, size_t smem);
+// launch shape of the grouped FP64 column kernel for nmem members of a size, false where it is not used
+bool colgroup_cfg(int nx, int ny, int nmem, int sms, LaunchCfg* c);
 template <class T> void set_row_smem_limits(int lim);
 template <class T> void set_col_smem_limits(int lim);
 // the column DFT of the low row modes of g (FP32 members): low_rows -> low_hat;

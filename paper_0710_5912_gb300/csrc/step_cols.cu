@@ -120,6 +120,52 @@ __device__ __forceinline__ void col_multiply_k(const ColConsts<T>& K, int m, T q
     }
   }
 }
+// The same for FP64 with every operation spelled out: k_colpass and k_colgroup
+// share it and must give the same bits, and the compiler contracts products by
+// their surroundings.
+template <int KIND>
+__device__ __forceinline__ void col_multiply_d(const ColConsts<double>& K, int m, double qx, double sqx, int nn,
+                                               double2& va, double2& vb) {
+  const int ns = nn < (K.ny >> 1) ? nn : nn - K.ny;
+  const double ky = __fma_rn((double)ns, K.qyu, -sqx);
+  const double k2 = __fma_rn(qx, qx, __dmul_rn(ky, ky));
+  const bool nyq_row = nn == (K.ny >> 1);
+  const double norm = K.norm;
+  if (KIND == 0) {
+    const double2 P = va, F = vb;
+    if (nyq_row) {
+      va = double2{__dmul_rn(-P.x, norm), __dmul_rn(-P.y, norm)};   // Nyquist row of phi^{n+1} -> 0
+    } else {
+      const double c4 = __dmul_rn(K.ckM, __dmul_rn(k2, k2));
+      const double aa = __fma_rn(K.caM, k2, -2.0 * c4);
+      const double bbm = __dmul_rn(K.cbM, k2);
+      const double inv = norm / (1.0 + c4);
+      va = double2{__dmul_rn(__fma_rn(aa, P.x, -__dmul_rn(bbm, F.x)), inv),
+                   __dmul_rn(__fma_rn(aa, P.y, -__dmul_rn(bbm, F.y)), inv)};
+    }
+    return;
+  }
+  const bool zero = nyq_row || (m == 0 && nn == 0);
+  const double2 G = va;
+  if (KIND == 2) {
+    const double inv = zero ? 0.0 : norm / __dmul_rn(k2, k2);
+    va = double2{__dmul_rn(G.x, inv), __dmul_rn(G.y, inv)};
+    return;
+  }
+  const double2 W = vb;
+  if (zero) {
+    va = double2{0.0, 0.0};
+    vb = double2{__dmul_rn(-W.x, norm), __dmul_rn(-W.y, norm)};     // omega^{n+1} -> 0 there
+  } else {
+    const double cc = __dmul_rn(K.cnu, k2), c2 = -2.0 * cc;
+    const double inv = 1.0 / (1.0 + cc);
+    const double2 dw = double2{__dmul_rn(__fma_rn(c2, W.x, __dmul_rn(K.dt, G.x)), inv),
+                               __dmul_rn(__fma_rn(c2, W.y, __dmul_rn(K.dt, G.y)), inv)};
+    const double ik = norm / k2;
+    va = double2{__dmul_rn(W.x + dw.x, ik), __dmul_rn(W.y + dw.y, ik)};
+    vb = double2{__dmul_rn(dw.x, norm), __dmul_rn(dw.y, norm)};
+  }
+}
 // FP32 inertial members: omega carried in 2D spectral form (w_hat).  At mode
 // (m, row nn): va = g_hat, vb = the transform of the advective increment A,
 // Wn = omega_hat^n (relabelled at a wrap).  omega* = Wn + A and Eq. forOmega
@@ -161,12 +207,11 @@ __device__ __forceinline__ void low_override(const MemberDesc& D, int m, int nn,
 }
 
 // the same with the kind chosen at run time (mode 0 or 1, and K.stokes)
-template <class T>
-__device__ __forceinline__ void col_multiply(int mode, const ColConsts<T>& K, int m, T qx, T sqx, int nn,
-                                             cplx<T>& va, cplx<T>& vb) {
-  if (mode == 0) col_multiply_k<0>(K, m, qx, sqx, nn, va, vb);
-  else if (K.stokes) col_multiply_k<2>(K, m, qx, sqx, nn, va, vb);
-  else col_multiply_k<1>(K, m, qx, sqx, nn, va, vb);
+__device__ __forceinline__ void col_multiply(int mode, const ColConsts<double>& K, int m, double qx, double sqx, int nn,
+                                             double2& va, double2& vb) {
+  if (mode == 0) col_multiply_d<0>(K, m, qx, sqx, nn, va, vb);
+  else if (K.stokes) col_multiply_d<2>(K, m, qx, sqx, nn, va, vb);
+  else col_multiply_d<1>(K, m, qx, sqx, nn, va, vb);
 }
 
 template <class T, int LN>
@@ -227,7 +272,7 @@ __global__ void __launch_bounds__(512, min_ctas<T>()) k_colpass(const MemberDesc
     T qx, sqx;
     K.mode_qx(mm, qx, sqx);
 #pragma unroll
-    for (int q = 0; q < kP; ++q) col_multiply<T>(mode, K, mm, qx, sqx, t + q * Tc, va[q], vb[q]);
+    for (int q = 0; q < kP; ++q) col_multiply(mode, K, mm, qx, sqx, t + q * Tc, va[q], vb[q]);
     fft_reg<true>(va, log2ny, t, buf, tws);
     if (active) {
 #pragma unroll
@@ -631,6 +676,105 @@ __global__ void __launch_bounds__(256, 2) k_colpass_single(const MemberDesc* __r
   else colpass_single_body<LN, 1>(D, log2nx, tw, smem_raw);
 }
 
+// The FP64 column pass of grids too small to fill the chip with one thread
+// group per mode: a CTA takes nm modes, and each input field of a mode is a
+// group of its own (threadIdx.y), so the two forward transforms, and for the
+// flow the two inverse ones, run side by side.  Columns are read straight into
+// the register layout and written from it (such grids live in L2, and each CTA
+// has one item: staging would only add latency); the fields meet once, through
+// their exchange buffers, for the multiplier.  What bounds it is the latency of
+// that chain and one warp's rate on an SM's FP64 pipe.  Kinds: 0 phi, 1 inertial
+// flow, 2 Stokes flow, 3 mixed (chosen per CTA).
+template <int LN, int KIND>
+__device__ __forceinline__ void colgroup_body(const MemberDesc& D, const double2* __restrict__ tw,
+                                              unsigned char* smem_raw) {
+  using C = double2;
+  constexpr int P = kP, ny = 1 << LN, Tc = ny / P;
+  constexpr bool two = KIND == 0 || KIND == 1;
+  const int nm = blockDim.x / Tc;
+  const int sub = threadIdx.x / Tc, t = threadIdx.x - sub * Tc, f = threadIdx.y;
+  const int m = blockIdx.x * nm + sub;
+  C* buf = reinterpret_cast<C*>(smem_raw) + (size_t)(f * nm + sub) * padded_len(ny);
+  C* other = reinterpret_cast<C*>(smem_raw) + (size_t)((1 - f) * nm + sub) * padded_len(ny);
+  C* tws = reinterpret_cast<C*>(smem_raw) + (size_t)blockDim.y * nm * padded_len(ny);
+  // a field's groups of whole warps synchronise alone, smaller ones together
+  const NamedSync sync = Tc >= 32 ? NamedSync{1 + f * nm + sub, Tc} : NamedSync{1 + f, (int)blockDim.x};
+  stage_tables_to_smem(tws, tw, LN, kLogP, f * blockDim.x + threadIdx.x, blockDim.x * blockDim.y);
+  __syncthreads();
+  pdl_wait();
+  if (!two && f == 1) return;                          // a Stokes member among inertial ones has one field
+  C* in = static_cast<C*>(KIND == 0 ? (f ? D.xs_f : D.xs_phi) : (f ? D.xs_w : D.xs_g)) + (size_t)m * ny;
+  C v[P];
+#pragma unroll
+  for (int q = 0; q < P; ++q) v[q] = in[t + q * Tc];
+  const ColConsts<double> K(D, KIND == 0 ? 0 : 1, ny);
+  double qx, sqx;
+  K.mode_qx(m, qx, sqx);
+  fft_reg<false>(v, LN, t, buf, tws, sync);
+  if constexpr (two) {
+#pragma unroll
+    for (int q = 0; q < P; ++q) buf[pad16(t + q * Tc)] = v[q];
+    __syncthreads();                                   // both fields' spectra in place
+    if (KIND == 0 && f == 1) return;                   // one result: the other group transforms it back
+#pragma unroll
+    for (int q = 0; q < P; ++q) {                      // each group forms its own result only
+      C o = other[pad16(t + q * Tc)];
+      if (f == 0) col_multiply_d<KIND>(K, m, qx, sqx, t + q * Tc, v[q], o);
+      else col_multiply_d<KIND>(K, m, qx, sqx, t + q * Tc, o, v[q]);
+    }
+    if (KIND == 1) __syncthreads();                    // the buffers are read, the inverse may use them
+  } else {
+#pragma unroll
+    for (int q = 0; q < P; ++q) col_multiply_d<KIND>(K, m, qx, sqx, t + q * Tc, v[q], v[q]);
+  }
+  fft_reg<true>(v, LN, t, buf, tws, sync);
+#pragma unroll
+  for (int q = 0; q < P; ++q) in[t + q * Tc] = v[q];
+}
+template <int LN, int KIND>
+__global__ void __launch_bounds__(512, 1) k_colgroup(const MemberDesc* __restrict__ descs,
+                                                     const double2* __restrict__ tw) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const MemberDesc& D = descs[blockIdx.y];
+  if (KIND != 3) colgroup_body<LN, KIND>(D, tw, smem_raw);
+  else if (D.stokes) colgroup_body<LN, 2>(D, tw, smem_raw);
+  else colgroup_body<LN, 1>(D, tw, smem_raw);
+}
+template <int LN>
+const void* colgroup_fn(int kind) {
+  if constexpr (2 * ((1 << LN) / kP) > 512) {
+    return nullptr;
+  } else {
+    switch (kind) {
+      case 0: return (const void*)k_colgroup<LN, 0>;
+      case 1: return (const void*)k_colgroup<LN, 1>;
+      case 2: return (const void*)k_colgroup<LN, 2>;
+      default: return (const void*)k_colgroup<LN, 3>;
+    }
+  }
+}
+// Launch shape of k_colgroup for a class, or false where k_colpass takes it.
+// Modes per CTA: whole warps.  The line: all modes' groups of both fields at
+// 256 threads per SM; beyond it the FP64 pipe is busy and k_colpass, which
+// stages the next column during a transform, is as fast.
+bool colgroup_cfg(int nx, int ny, int nmem, int sms, LaunchCfg* c) {
+  const int Tc = ny / kP;
+  int nm = 1;
+  while (nm * Tc < 32) nm *= 2;
+  if (2 * nm * Tc > 512 || nm > nx / 2) return false;
+  if ((long long)(nx / 2) * 2 * Tc * nmem > 256ll * sms) return false;
+  int log2ny = 0;
+  while ((1 << log2ny) < ny) ++log2ny;
+  c->grid_x = (nx / 2) / nm;
+  c->grid_y = 1;
+  c->threads = nm * Tc;
+  c->groups = 2;
+  c->inst_per_cta = nm;
+  c->variant = 0;
+  c->smem = 2 * (size_t)nm * padded_len(ny) * sizeof(double2) + stage_table_bytes(log2ny, kLogP, sizeof(double));
+  return true;
+}
+
 // the FP32 column kernels of a length: the chunk kernel for ny >= 512, else
 // the single-mode kernel
 template <int LN>
@@ -670,6 +814,12 @@ void launch_col_kernel(int kind, const MemberDesc* d, int nmem, int log2nx, int 
       void* args[] = {(void*)&dd, (void*)&log2nx, (void*)&tt};
       launch_pdl(colpass_fp32_fn<LN>(k), grid, c.threads, args, c.smem, st);
     } else {
+      if (c.groups > 1) {
+        const int k = mode == 0 ? 0 : (c.variant >= 1 && c.variant <= 3 ? c.variant : 3);
+        void* args[] = {(void*)&d, (void*)&tw};
+        launch_pdl(colgroup_fn<LN>(k), grid, dim3(c.threads, k == 2 ? 1 : 2), args, c.smem, st);
+        return;
+      }
       void* args[] = {(void*)&d, (void*)&log2nx, (void*)&tw, (void*)&mode};
       launch_pdl((const void*)k_colpass<T, LN>, grid, c.threads, args, c.smem, st);
     }
@@ -697,8 +847,11 @@ void set_col_smem_limits(int lim) {
       if constexpr (sizeof(T) == 4) {
         for (int k = 0; k < 5; ++k)
           cudaFuncSetAttribute(colpass_fp32_fn<LN>(k), cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-      } else
+      } else {
         cudaFuncSetAttribute(k_colpass<T, LN>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+        for (int k = 0; k < 4; ++k)
+          if (colgroup_fn<LN>(k)) cudaFuncSetAttribute(colgroup_fn<LN>(k), cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+      }
     });
 }
 

@@ -38,7 +38,7 @@ __device__ __forceinline__ void low_row_terms(const float* stage, float* Zb, con
   float2 u[16];
 #pragma unroll
   for (int q = 0; q < 16; ++q) u[q] = float2{stage[t + q * Tc], stage[N + t + q * Tc]};
-  dft16<false>(u);                                     // u[r] = y_t[r]
+  dft16<false>(u);                            // u[r] = y_t[r]
   // W_N^t and W_N^{2t} (forward sign) from the last stage's pairs
   float2 w1 = float2{1.f, 0.f}, w2 = float2{1.f, 0.f};
   if (log2nx > 4) {
