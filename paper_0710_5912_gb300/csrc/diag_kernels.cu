@@ -285,14 +285,22 @@ __global__ void __launch_bounds__(512) k_sf_rows(const T* __restrict__ f, cplx<T
 // Partials per CTA (kSfMoments): sum S, sum k S, sum S/k, and for the tensor
 // of Eq. L_matrix sum q_cx^2 S, sum q_cx q_cy S, sum q_cy^2 S, sum S with
 // k = 0 included.
+// What bounds it is the FP64 pipe (16 cycles of an SM per warp instruction).  A
+// thread's eight modes lie in one column, so q_x leaves their sums; they are
+// added in pairs, and only the threads' totals are added with compensation, by
+// one warp per moment (six compensated sums of every mode and of every lane
+// took about 150 us of a 1024^2 pass).  For the bins: along a column k grows
+// away from ky = 0 on either side, so a bin's modes are one run on each, which
+// the bin's thread finds by bisection instead of looking at every mode.
 template <class T>
 __global__ void __launch_bounds__(512) k_sf_cols(const cplx<T>* __restrict__ xs, int log2nx, int log2ny,
                                                   double dx, double s, const cplx<T>* __restrict__ tw,
                                                   double* __restrict__ partials, int nbins,
                                                   double* __restrict__ bin_partials) {
   using C = cplx<T>;
+  constexpr int kSums = 6;                              // sum S, k S, S/k, qx^2 S, qx ky S, ky^2 S
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ double sh[2 * kSfMoments * 32];
+  __shared__ int first_up[512];                         // per column: the first row with ky >= 0
   const int nx = 1 << log2nx, ny = 1 << log2ny, half = nx >> 1;
   const int Tc = ny >> 3;
   const int col = threadIdx.x / Tc, tid = threadIdx.x - col * Tc;
@@ -306,15 +314,24 @@ __global__ void __launch_bounds__(512) k_sf_cols(const cplx<T>* __restrict__ xs,
     const int c = e & (ncol - 1), n = e >> log2ncol;
     sm[c * ny + n] = xs[(size_t)n * half + m0 + c];
   }
+  if (threadIdx.x < ncol) first_up[threadIdx.x] = ny >> 1;
   C* const b1[1] = {sm + col * ny};
   fft_smem<false, 1>(b1, log2ny, tid, tw);
   const int m = m0 + col;
   const double two_pi = 6.283185307179586476925286766559;
   const double qx = two_pi * m / (nx * dx);
   const double norm = 1.0 / ((double)nx * (double)ny);
-  const double dk = two_pi / (ny * dx);
-  double acc_s[kSfMoments], acc_c[kSfMoments];
-  for (int v = 0; v < kSfMoments; ++v) acc_s[v] = acc_c[v] = 0.0;
+  const double dk = two_pi / (ny * dx), inv_dk = 1.0 / dk;
+  // the lab wavenumber of row ns; a box of a power-of-two length divides exactly
+  const double Ly = ny * dx, inv_Ly = 1.0 / Ly;
+  const bool exact_inv = (__double_as_longlong(Ly) & 0xfffffffffffffll) == 0;
+  auto ky_of = [&](int ns) {
+    const double t = __dmul_rn(two_pi, (double)ns);
+    return __fma_rn(-s, qx, exact_inv ? __dmul_rn(t, inv_Ly) : t / Ly);
+  };
+  double v[kSums][2] = {};                              // two partial sums each (even and odd q)
+  double origin = 0.0;                                  // S of k = 0
+#pragma unroll
   for (int q = 0; q < 8; ++q) {
     const int n = tid + q * Tc;
     const int idx = col * ny + n;
@@ -322,52 +339,124 @@ __global__ void __launch_bounds__(512) k_sf_cols(const cplx<T>* __restrict__ xs,
     int b = -1;
     if (n != (ny >> 1)) {
       const int ns = n < (ny >> 1) ? n : n - ny;
-      const double qy = two_pi * ns / (ny * dx);
-      const double ky = qy - s * qx;
+      const double ky = ky_of(ns);
       const C X = sm[idx];
       const double re = (double)X.x * norm, im = (double)X.y * norm;
       const double S = (m == 0 ? 1.0 : 2.0) * (re * re + im * im);
-      neumaier_add(acc_s[3], acc_c[3], qx * qx * S);
-      neumaier_add(acc_s[4], acc_c[4], qx * ky * S);
-      neumaier_add(acc_s[5], acc_c[5], ky * ky * S);
-      neumaier_add(acc_s[6], acc_c[6], S);
-      if (!(m == 0 && n == 0)) {
-        const double k = sqrt(qx * qx + ky * ky);
-        neumaier_add(acc_s[0], acc_c[0], S);
-        neumaier_add(acc_s[1], acc_c[1], k * S);
-        neumaier_add(acc_s[2], acc_c[2], S / k);
-        w = S;
-        const double fb = floor(k / dk);
-        b = (fb < (double)nbins) ? (int)fb : -1;
+      if (m == 0 && n == 0) {
+        origin = S;
+        v[5][q & 1] += ky * ky * S;
+        b = 0;
+      } else {
+        const double k2 = __fma_rn(qx, qx, __dmul_rn(ky, ky));
+        const double rk = rsqrt(k2), k = k2 * rk;
+        v[0][q & 1] += S;
+        v[1][q & 1] += k * S;
+        v[2][q & 1] += S * rk;
+        v[4][q & 1] += ky * S;
+        v[5][q & 1] += ky * ky * S;
+        if (nbins > 0) {
+          w = S;
+          const double t = k * inv_dk;
+          double fb = floor(t);
+          if (t - fb < 1e-9 || t - fb > 1.0 - 1e-9) fb = floor(sqrt(k2) / dk);   // on an edge: the quotient decides
+          b = fb < (double)nbins ? (int)fb : nbins;
+        }
       }
+      if (nbins > 0 && ky >= 0.0 && (ns == 1 - (ny >> 1) || ky_of(ns - 1) < 0.0))
+        first_up[col] = ns;
     }
     if (nbins > 0) {
       Sw[idx] = w;
       bin[idx] = b;
     }
   }
-  block_reduce_pairs<kSfMoments>(acc_s, acc_c, sh);
-  if (threadIdx.x == 0) {
-    for (int v = 0; v < kSfMoments; ++v) partials[kSfMoments * blockIdx.x + v] = acc_s[v] + acc_c[v];
+  __syncthreads();                                      // the spectra are read: their place holds the threads' sums
+  double* part = reinterpret_cast<double*>(smem_raw);   // [sum][thread]
+  {
+    const double S0 = v[0][0] + v[0][1];
+    part[0 * blockDim.x + threadIdx.x] = S0;
+    part[1 * blockDim.x + threadIdx.x] = v[1][0] + v[1][1];
+    part[2 * blockDim.x + threadIdx.x] = v[2][0] + v[2][1];
+    part[3 * blockDim.x + threadIdx.x] = qx * qx * S0;
+    part[4 * blockDim.x + threadIdx.x] = qx * (v[4][0] + v[4][1]);
+    part[5 * blockDim.x + threadIdx.x] = v[5][0] + v[5][1];
   }
-  if (nbins > 0) {
-    __syncthreads();
-    for (int bb = threadIdx.x; bb < nbins; bb += blockDim.x) {
+  __syncthreads();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  double* out = partials + kSfMoments * blockIdx.x;
+  if (nw == 0) {                                        // the smallest grids: fewer threads than a warp
+    for (int j = threadIdx.x; j < kSums; j += blockDim.x) {
       double sum = 0.0, comp = 0.0;
-      for (int e = 0; e < ncol * ny; ++e)
-        if (bin[e] == bb) neumaier_add(sum, comp, Sw[e]);
-      bin_partials[(size_t)blockIdx.x * nbins + bb] = sum + comp;
+      for (int i = 0; i < blockDim.x; ++i) neumaier_add(sum, comp, part[j * blockDim.x + i]);
+      out[j] = sum + comp;
+      if (j == 0) out[6] = sum + comp;
     }
+    __syncthreads();
+    if (threadIdx.x == 0 && m0 == 0) out[6] += origin;
+  } else {
+    for (int j = warp; j < kSums; j += nw) {
+      double sum = 0.0, comp = 0.0;
+      for (int i = lane; i < blockDim.x; i += 32) neumaier_add(sum, comp, part[j * blockDim.x + i]);
+#pragma unroll
+      for (int off = 16; off > 0; off >>= 1) {
+        const double os = __shfl_down_sync(0xffffffffu, sum, off), oc = __shfl_down_sync(0xffffffffu, comp, off);
+        if (lane < off) {
+          neumaier_add(sum, comp, os);
+          comp += oc;
+        }
+      }
+      if (lane == 0) {
+        out[j] = sum + comp;
+        // with k = 0, which thread 0 (lane 0 of warp 0, so j = 0 here) holds
+        if (j == 0) {
+          neumaier_add(sum, comp, origin);
+          out[6] = sum + comp;
+        }
+      }
+    }
+  }
+  for (int bb = threadIdx.x; bb < nbins; bb += blockDim.x) {
+    double sum = 0.0, comp = 0.0;
+    for (int c = 0; c < ncol; ++c) {
+      const int up = first_up[c];
+#pragma unroll
+      for (int side = 0; side < 2; ++side) {
+        // place i of the side: row up + i (ky >= 0) or up - 1 - i (ky < 0)
+        const int count = side == 0 ? (ny >> 1) - up : up + (ny >> 1) - 1;
+        const int* bc = bin + c * ny;
+        auto row = [&](int i) { return (side == 0 ? up + i : up - 1 - i) & (ny - 1); };
+        if (count <= 0 || bc[row(0)] > bb || bc[row(count - 1)] < bb) continue;
+        int lo = 0, hi = count;
+        while (lo < hi) {                               // the first place whose bin is not below bb
+          const int mid = (lo + hi) >> 1;
+          if (bc[row(mid)] < bb) lo = mid + 1;
+          else hi = mid;
+        }
+        for (; lo < count && bc[row(lo)] == bb; ++lo) neumaier_add(sum, comp, Sw[c * ny + row(lo)]);
+      }
+    }
+    bin_partials[(size_t)blockIdx.x * nbins + bb] = sum + comp;
   }
 }
 
-// Column sums of a rows x cols array, each column summed over rows in order.
+// Column sums of a rows x cols array: one warp per column, its lanes over
+// every 32nd row in order, then a fixed tree (a single thread's chain of
+// compensated FP64 additions over 128..2048 rows took longer than the sums).
 __global__ void k_reduce_rows(const double* __restrict__ in, int rows, int cols, double* __restrict__ out) {
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= cols) return;
+  const int c = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+  if (c >= cols) return;                               // whole warps
   double sum = 0.0, comp = 0.0;
-  for (int r = 0; r < rows; ++r) neumaier_add(sum, comp, in[(size_t)r * cols + c]);
-  out[c] = sum + comp;
+  for (int r = lane; r < rows; r += 32) neumaier_add(sum, comp, in[(size_t)r * cols + c]);
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) {
+    const double os = __shfl_down_sync(0xffffffffu, sum, off), oc = __shfl_down_sync(0xffffffffu, comp, off);
+    if (lane < off) {
+      neumaier_add(sum, comp, os);
+      comp += oc;
+    }
+  }
+  if (lane == 0) out[c] = sum + comp;
 }
 
 // ----------------------------------------------------------------- launchers
@@ -413,7 +502,7 @@ void launch_sf_cols(const cplx<T>* xs, int log2nx, int log2ny, double dx, double
                                                   bin_partials);
 }
 void launch_reduce_rows(const double* in, int rows, int cols, double* out, cudaStream_t st) {
-  k_reduce_rows<<<(cols + 127) / 128, 128, 0, st>>>(in, rows, cols, out);
+  k_reduce_rows<<<(cols + 3) / 4, 128, 0, st>>>(in, rows, cols, out);
 }
 
 template <class T>
