@@ -257,7 +257,7 @@ LaunchCfg persistent_cfg(int kind, int nfft, int max_inst, int items, size_t ins
 
 // Thread groups per CTA of the forward row passes (stage 1: up to three, one
 // per transform of an item; stage 2: two, the transform and the low row
-// modes).  One group's transforms follow one another in the item's threads,
+// modes, in FP64 up to four, which share the stencil).  One group's transforms follow one another in the item's threads,
 // which keeps a full chip busy; where the row pairs of a launch are too few for
 // that, the groups run them side by side and share the stencil: as long as all
 // pairs' groups fit on the chip at once (768 threads per SM at 80 registers;
@@ -295,7 +295,7 @@ void configure_class_t(SizeClass& cl, Tune tune) {
   const int nx = cl.nx, ny = cl.ny, nmem = (int)cl.members.size();
   // (a pair of groups only would leave inertial members a transform behind)
   const int g1 = stage_groups<T>(3, nx, ny, nmem, tune.stage1_points) == 3 ? 3 : 1;
-  const int g2 = stage_groups<T>(2, nx, ny, nmem, tune.stage2_points);
+  const int g2 = stage_groups<T>(R == 8 ? 4 : 2, nx, ny, nmem, tune.stage2_points);
   cl.cfg[KIND_STAGE1] = persistent_cfg<T>(KIND_STAGE1, nx, ny / 2, ny / 2, (g1 > 1 ? 3 : 2) * stage1_inst_bytes(nx, R), nmem,
                                            tune.stage1_points, 0, g1);
   cl.cfg[KIND_STAGE2] = persistent_cfg<T>(KIND_STAGE2, nx, ny / 2, ny / 2, rowfwd_inst_bytes(nx, R, g2), nmem,

@@ -121,9 +121,10 @@ __device__ __forceinline__ void strain_dev(long long n, double gdot_dt, double r
 // one x-spectral chunk column of each input field plus the buffer; rowinv
 // stages the 32-byte chunks of a row pair (nx complex) plus the buffer.
 __host__ __device__ constexpr size_t round128(size_t b) { return (b + 127) & ~(size_t)127; }
-// (with several groups a second buffer for the low modes' terms)
+// (with several groups a second buffer for the low modes' terms, in FP64 for mu)
 __host__ __device__ constexpr size_t rowfwd_inst_bytes(int nx, size_t real_bytes, int groups) {
-  return round128(2 * (size_t)nx * real_bytes + (groups > 1 ? 2 : 1) * (size_t)padded_len(nx) * 2 * real_bytes);
+  return round128(2 * (size_t)nx * real_bytes +
+                  (groups > 1 || real_bytes == 8 ? 2 : 1) * (size_t)padded_len(nx) * 2 * real_bytes);
 }
 // the FP64 column pass stages two columns of 16-byte complex doubles plus
 // the padded exchange buffer

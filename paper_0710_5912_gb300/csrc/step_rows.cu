@@ -217,6 +217,83 @@ __device__ __forceinline__ void stage2_pair(const MemberDesc& D, const T* __rest
   }
 }
 
+// The same for FP64, in two passes over the item: mu of rows j0 - 1 .. j0 + 2
+// into shared memory (rows 0, 1 in mu01, 2, 3 in mu23, nx reals each), and after
+// a barrier the curl from it.  The FP64 pipe bounds this pass: the register
+// windows above form each mu four times (two rows' and two neighbours' worth),
+// this once per row pair that needs it, 46 FP64 instructions per point instead
+// of 72, and the windows spilled 436 bytes per thread.  The caller's barrier
+// comes between the two halves.  (Products are spelled out: the two thread
+// groupings must give the same bits.)
+__device__ __forceinline__ void stage2_mu_f64(const MemberDesc& D, const double* __restrict__ phi, double* mu01,
+                                              double* mu23, int j0, int log2nx, int my, const Shear<double>& sc, int t,
+                                              int Tf) {
+  const int nx = 1 << log2nx, mx = nx - 1;
+  const RealPar<double>& p = D.d;
+  const double kxx = __dmul_rn(__dmul_rn(p.kappa, __fma_rn(sc.s, sc.s, 1.0)), p.inv_h2);
+  const double kxy = __dmul_rn(__dmul_rn(p.kappa, 2.0 * sc.s), p.inv_4h2), kyy = __dmul_rn(p.kappa, p.inv_h2);
+  for (int q = t; q < (nx >> 2); q += Tf) {
+    const int x0 = 4 * q;
+    auto row6 = [&](int j) {                           // columns x0 - 1 .. x0 + 4
+      const double* r = phi + ((size_t)(j & my) << log2nx);
+      const Quad<double> c = ldg4(r + x0);
+      return Six<double>{{__ldg(r + ((x0 - 1) & mx)), c.v[0], c.v[1], c.v[2], c.v[3], __ldg(r + ((x0 + 4) & mx))}};
+    };
+    Six<double> Dn = row6(j0 - 2), C = row6(j0 - 1);
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      const Six<double> U = row6(j0 + r);
+      double m[4];
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        const double pc = C.v[c + 1];
+        const double sxx = __fma_rn(-2.0, pc, C.v[c + 2]) + C.v[c];
+        const double syy = __fma_rn(-2.0, pc, U.v[c + 1]) + Dn.v[c + 1];
+        const double sxy = (U.v[c + 2] - Dn.v[c + 2]) - (U.v[c] - Dn.v[c]);
+        const double klap = __fma_rn(kyy, syy, __fma_rn(kxx, sxx, -__dmul_rn(kxy, sxy)));
+        m[c] = __fma_rn(pc, __fma_rn(p.b, __dmul_rn(pc, pc), -p.a), -klap);
+      }
+      st4((r < 2 ? mu01 : mu23) + (r & 1) * nx + x0, m[0], m[1], m[2], m[3]);
+      Dn = C;
+      C = U;
+    }
+  }
+}
+template <bool NEG>
+__device__ __forceinline__ void stage2_curl_f64(const MemberDesc& D, const double* __restrict__ phi, const double* mu01,
+                                                const double* mu23, double* buf, int j0, int log2nx, int my,
+                                                const Shear<double>& sc, int t, int Tf) {
+  const int nx = 1 << log2nx, mx = nx - 1;
+  // the derivatives' 1 / 2h of both factors and c_force in one product
+  const double scale = __dmul_rn(D.d.c_force, __dmul_rn(D.d.inv_2h, D.d.inv_2h));
+  auto mu_row = [&](int r) { return (r < 2 ? mu01 : mu23) + (r & 1) * nx; };
+  auto row8 = [&](const double* r, int x0) {           // columns x0 - 2 .. x0 + 5
+    const double2 l = *reinterpret_cast<const double2*>(r + ((x0 - 2) & mx)), e = *reinterpret_cast<const double2*>(r + ((x0 + 4) & mx));
+    const Quad<double> c = ld4(r + x0);
+    return Row8<double>{{l.x, l.y, c.v[0], c.v[1], c.v[2], c.v[3], e.x, e.y}};
+  };
+  for (int q = t; q < (nx >> 2); q += Tf) {
+    const int x0 = 4 * q;
+    auto prow = [&](int j) { return row8(phi + ((size_t)(j & my) << log2nx), x0); };
+    Row8<double> pD = prow(j0 - 1), pC = prow(j0), mD = row8(mu_row(0), x0), mC = row8(mu_row(1), x0);
+#pragma unroll
+    for (int o = 0; o < 2; ++o) {
+      const Row8<double> pU = prow(j0 + o + 1), mU = row8(mu_row(o + 2), x0);
+      double r[4];
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        auto dy = [&](const Row8<double>& U, const Row8<double>& Dn) {
+          const double up = NEG ? U.v[c + 4] : U.v[c], dn = NEG ? Dn.v[c] : Dn.v[c + 4];
+          return __fma_rn(sc.w0, U.v[c + 2] - Dn.v[c + 2], __dmul_rn(sc.w1, up - dn));
+        };
+        r[c] = __dmul_rn(scale, diff_of_products(pC.v[c + 3] - pC.v[c + 1], dy(mU, mD), dy(pU, pD), mC.v[c + 3] - mC.v[c + 1]));
+      }
+      st4(buf + o * nx + x0, r[0], r[1], r[2], r[3]);
+      pD = pC; pC = pU; mD = mC; mC = mU;
+    }
+  }
+}
+
 // ====================================================== forward row transforms
 // Work items: one per row pair p = rows (2p, 2p+1).  Mode 1 is stage 2: the
 // stage-2 stencil of the pair (stage2_pair) computed straight into the
@@ -281,8 +358,19 @@ __global__ void __launch_bounds__(rows_max_threads<T>(P, GROUPED), rows_min_ctas
     const int p = w;
     if constexpr (MODE == 1) {
       const int j0 = 2 * (active ? w : 0);
-      if (sc.d > 0) stage2_pair<true>(D, src, stage, j0, log2nx, my, sc, grp * Tf + t, G * Tf);
-      else stage2_pair<false>(D, src, stage, j0, log2nx, my, sc, grp * Tf + t, G * Tf);
+      const int ts = grp * Tf + t, Ts = G * Tf;          // this thread's place in the stencil
+      if constexpr (sizeof(T) == 8) {
+        T* mu01 = reinterpret_cast<T*>(Z);              // the exchange buffer and the one behind it
+        T* mu23 = reinterpret_cast<T*>(Z + padded_len(nx));
+        if (it > 0) __syncthreads();                    // group 0 is done with the buffers
+        stage2_mu_f64(D, src, mu01, mu23, j0, log2nx, my, sc, ts, Ts);
+        __syncthreads();
+        if (sc.d > 0) stage2_curl_f64<true>(D, src, mu01, mu23, stage, j0, log2nx, my, sc, ts, Ts);
+        else stage2_curl_f64<false>(D, src, mu01, mu23, stage, j0, log2nx, my, sc, ts, Ts);
+      } else {
+        if (sc.d > 0) stage2_pair<true>(D, src, stage, j0, log2nx, my, sc, ts, Ts);
+        else stage2_pair<false>(D, src, stage, j0, log2nx, my, sc, ts, Ts);
+      }
       __syncthreads();                                 // the pair's g complete
       prefetch(w + stride);                            // the next item's rows, during the transform
     } else {
