@@ -131,6 +131,7 @@ struct shf_grid {
   std::vector<cudaEvent_t> joins;            // ensembles: the grid's stream waits on them
   cudaEvent_t phi_done = nullptr;     // recorded after the last step's phi row inverse
   bool what_valid = false;            // FP32: w_hat holds the 2D transform of the current omega
+  bool state_valid = false;           // the members' StepState is step n's: the last step left it so
   std::vector<shf_grid*> views;
   std::string err;
 };
@@ -403,6 +404,8 @@ MemberDesc make_desc(const shf_grid* o, const Member& m) {
 }
 
 int upload_desc(shf_grid* o, int mi) {
+  o->state_valid = false;   // the next run starts with a plain launch, ordered behind this copy (step kernels
+                            // read descriptors before they wait for their predecessor)
   Member& m = o->members[mi];
   SizeClass& cl = o->classes[m.cls];
   cl.h_desc[m.slot] = make_desc(o, m);
@@ -702,13 +705,17 @@ void enqueue_step(shf_grid* o) {
     for (int k = 0; k < kKinds; ++k) launch_kind<T>(o, cl, k);
 }
 
-// every member's StepState from its counter; needed once before a run of
-// steps (each step's last kernel then prepares the next step's state).  FP32
+// every member's StepState from its counter, where the last step has not left
+// it (each step's last kernel prepares the next step's; a new grid, new
+// parameters, a set counter or a failed wait call for it: 4 us of a single step
+// per call).  FP32
 // grids whose fields were set from outside since their last step also get
 // w_hat, omega's 2D transform, recomputed from omega (a row pass and a column
 // pass; members without w_hat skip them).
 void enqueue_state_init(shf_grid* o) {
-  for (auto& cl : o->classes) launch_step_state_init(cl.d_desc, (int)cl.members.size(), o->stream);
+  if (!o->state_valid)
+    for (auto& cl : o->classes) launch_step_state_init(cl.d_desc, (int)cl.members.size(), o->stream);
+  o->state_valid = true;
   if (o->precision == SHF_FP32 && !o->what_valid) {
     for (auto& cl : o->classes) {
       const int nm = (int)cl.members.size();
@@ -1316,6 +1323,7 @@ int shf_set_step(shf_grid* g, int64_t n) {
   SHF_CUDA(g, cudaStreamSynchronize(g->stream));
   g->n = n;
   g->what_valid = false;                                // the next step re-reads omega
+  g->state_valid = false;
   return SHF_OK;
 }
 
@@ -1468,6 +1476,7 @@ int shf_sync(shf_grid* g) {
   SHF_CUDA(g, cudaMemcpy(&err, o->d_err, sizeof(int), cudaMemcpyDeviceToHost));
   if (err) {
     SHF_CUDA(g, cudaMemset(o->d_err, 0, sizeof(int)));
+    o->state_valid = false;
     return fail(g, SHF_ETIMEOUT, "a kernel's bounded wait for its input copies gave up");
   }
   std::vector<int> which;
