@@ -130,6 +130,7 @@ struct shf_grid {
   cudaEvent_t fork = nullptr;                // ensembles: class streams wait on it
   std::vector<cudaEvent_t> joins;            // ensembles: the grid's stream waits on them
   cudaEvent_t phi_done = nullptr;     // recorded after the last step's phi row inverse
+  cudaEvent_t in_done = nullptr;      // shf_step_host_f32: phi and psi have arrived
   bool what_valid = false;            // FP32: w_hat holds the 2D transform of the current omega
   bool state_valid = false;           // the members' StepState is step n's: the last step left it so
   std::vector<shf_grid*> views;
@@ -490,6 +491,7 @@ void free_all(shf_grid* g) {
   cudaFree(g->d_scratch);
   if (g->h_pinned) cudaFreeHost(g->h_pinned);
   if (g->phi_done) cudaEventDestroy(g->phi_done);
+  if (g->in_done) cudaEventDestroy(g->in_done);
   if (g->io_stream) cudaStreamDestroy(g->io_stream);
   for (auto st : g->class_streams) cudaStreamDestroy(st);
   for (auto ev : g->joins) cudaEventDestroy(ev);
@@ -1347,14 +1349,30 @@ int shf_step_host_f32(shf_grid* g, int64_t nsteps, const float* phi_in, const fl
   SHF_CUDA(g, cudaSetDevice(g->device));
   if (!g->io_stream) SHF_CUDA(g, cudaStreamCreateWithFlags(&g->io_stream, cudaStreamNonBlocking));
   if (!g->phi_done) SHF_CUDA(g, cudaEventCreateWithFlags(&g->phi_done, cudaEventDisableTiming));
+  if (!g->in_done) SHF_CUDA(g, cudaEventCreateWithFlags(&g->in_done, cudaEventDisableTiming));
   const size_t bytes = (size_t)m.nx * m.ny * sizeof(float);
   if (phi_in) {
     g->what_valid = false;
     const float* src[3] = {phi_in, psi_in, m.rho > 0 ? omega_in : nullptr};
     void* dst[3] = {m.phi, m.psi, m.omega};
-    for (int f = 0; f < 3; ++f) {
-      if (src[f]) SHF_CUDA(g, cudaMemcpyAsync(dst[f], src[f], bytes, cudaMemcpyHostToDevice, g->stream));
-      else SHF_CUDA(g, cudaMemsetAsync(dst[f], 0, bytes, g->stream));
+    // an inertial run transforms omega before its first step (w_hat): omega
+    // goes first and is transformed while phi and psi cross the link on the
+    // second stream, behind what the grid's stream still does
+    const bool ahead = nsteps > 0 && src[2];
+    cudaStream_t st = ahead ? g->io_stream : g->stream;
+    if (ahead) {
+      SHF_CUDA(g, cudaEventRecord(g->phi_done, g->stream));
+      SHF_CUDA(g, cudaStreamWaitEvent(g->io_stream, g->phi_done, 0));
+    }
+    for (int f = 2; f >= 0; --f) {
+      cudaStream_t s = f == 2 ? g->stream : st;
+      if (src[f]) SHF_CUDA(g, cudaMemcpyAsync(dst[f], src[f], bytes, cudaMemcpyHostToDevice, s));
+      else SHF_CUDA(g, cudaMemsetAsync(dst[f], 0, bytes, s));
+    }
+    if (ahead) {
+      SHF_CUDA(g, cudaEventRecord(g->in_done, g->io_stream));
+      enqueue_state_init(g);
+      SHF_CUDA(g, cudaStreamWaitEvent(g->stream, g->in_done, 0));
     }
   }
   const bool early = nsteps > 0 && phi_out;
