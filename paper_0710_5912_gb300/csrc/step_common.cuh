@@ -104,6 +104,7 @@ __device__ __forceinline__ F2 df_add(F2 a, F2 b) {
   const F2 s = two_sum_f(a.hi, b.hi);
   return fast_two_sum_f(s.hi, __fadd_rn(s.lo, __fadd_rn(a.lo, b.lo)));
 }
+__device__ __forceinline__ F2 df_neg(F2 a) { return F2{-a.hi, -a.lo}; }
 __device__ __forceinline__ F2 df_mul(F2 a, F2 b) {
   const float p = __fmul_rn(a.hi, b.hi);
   float e = __fmaf_rn(a.hi, b.hi, -p);

@@ -68,66 +68,42 @@ __global__ void k_step_state_init(const MemberDesc* __restrict__ descs, int nmem
 // need F itself beyond FP32.  This kernel forms, for members with D.low == 2
 // (FP32 Stokes), the row DFT coefficients m = 0..lowm of
 //   g = c_force (D_x phi D_y^s mu - D_y^s phi D_x mu)
-// with F evaluated in double-float from the FP32 phi^{n+1} and an FP32 mu: the differences of two FP32 values
+// with F evaluated in double-float from the FP32 phi^{n+1} and an FP32 mu
+// (mu as the stage-2 stencil forms it): the differences of two FP32 values
 // are exact as pairs, the Eq. p1y weights w0 = 1 - |s|/2, w1 = |s|/2 come from
 // the FP64 strain, and every product and sum carries its rounding error.
 // The DFT terms F W^{m x} use the double-float twiddle table and are summed
 // as double-float pairs; the threads' sums are folded in a fixed order.  The
 // result, hi and lo planes of low_rows, feeds k_lowmode_cols like the
 // compensated sums of the row pass do for the other FP32 members.
-// Work: a CTA takes 32 rows and XT columns of the first quarter of the rows,
-// with the same columns shifted by one, two and three quarters: since
-// W^{m (x + nx/4)} = (-i)^m W^{m x}, the four are folded before the DFT.  With
-// E, O = F(x) +- F(x + nx/2) and E', O' the same a quarter further, the terms are
-// (E + E') W^{mx} for m = 0, 4, 8, (E - E') W^{mx} for m = 2, 6 and
-// (O -+ i O') W^{mx} for odd m: 24 real products per four points where folding
-// halves alone takes 32.  phi (halo 2 rows, 3 columns) and mu (halo 1 row, 2
-// columns) of the four tiles sit in shared memory; lane r of every warp owns
+// Work: a CTA takes up to 32 rows x 64 columns of the first half of the rows
+// and the same columns shifted by nx / 2, folded before the DFT: since
+// W^{m (x + nx/2)} = (-1)^m W^{m x}, the terms of both are
+// (F(x) + F(x + nx/2)) W^{m x} for even m and (F(x) - F(x + nx/2)) W^{m x}
+// for odd m, half the products.  phi (halo 2 rows, 3 columns) and mu (halo 1
+// row, 2 columns) of both tiles sit in shared memory; lane r of every warp owns
 // row j0 + r and its warp's slice of the columns, so a thread sums its own row
-// and the twiddle W^{m x} is the same for the whole warp (one broadcast load).
-// The 8 warps' sums of a row are folded in warp order; with several column
-// tiles per row the CTAs park their sums in a scratch area and the last CTA of
-// a row block to finish (an atomic counter; nothing waits) folds them in tile
-// order into low_rows and scales them (c_force / 4 h^2, once per sum instead of
-// once per point).  What bounds it is FP32 issue: about 230 instructions per
-// point, 84 of them F and 75 the DFT's sums; pairs are renormalised only where
-// a sum needs it.  Four CTAs per SM (64 registers): 210 us at 4096^2, where
-// three took 232, two 303, and the tiles of two halves and 118-instruction F
-// with runtime-divided indices 350.  XT is 32, or less where that makes fewer
-// than 200 CTAs: with the column DFT, 1024^2 31.3 us (XT = 16: 36.8), 1024 x 512
-// 29.3 -> 27.2 at 16, 512^2 26.9 -> 22.2 at 8, 128^2 21.1 -> 16.6 at 8.
+// and the twiddle W^{m x} is the same for the whole warp (one broadcast load).  The 8 warps' sums of a row are folded in
+// warp order; with several column tiles per row the CTAs park their sums in
+// a scratch area and the last CTA of a row block to finish (an atomic
+// counter; nothing waits) folds them in tile order into low_rows.
 constexpr int kLxRows = 32;     // rows per CTA: one per lane
+constexpr int kLxCols = 64;     // columns per CTA
 constexpr int kLxWarps = 8;
 constexpr int kLxValues = 2 * (kLowMExact + 1);   // Re and Im of m = 0..kLowMExact
+// a CTA's tile covers XT columns of the first half of the rows and the same
+// columns shifted by nx / 2 (the DFT folds them: W^{m (x + nx/2)} = (-1)^m W^{m x})
+__host__ __device__ constexpr int lowexact_cols(int nx) { return nx / 2 < kLxCols ? nx / 2 : kLxCols; }
 __host__ __device__ constexpr int lowexact_rows(int ny) { return ny < kLxRows ? ny : kLxRows; }
-// columns per quarter (from the size alone: the order of the sums depends on it)
-inline int lowexact_cols(int nx, int ny) {
-  int xt = nx / 4 < 32 ? nx / 4 : 32;
-  while (xt > 8 && (nx / 4 / xt) * (ny / lowexact_rows(ny)) < 200) xt /= 2;
-  return xt;
-}
 __host__ __device__ constexpr int lowexact_pitch_phi(int xt) { return (xt + 6) | 1; }
 __host__ __device__ constexpr int lowexact_pitch_mu(int xt) { return (xt + 4) | 1; }
-__host__ __device__ constexpr int lowexact_tile_floats(int xt, int rt) {   // one phi tile and its mu tile
-  return (rt + 4) * lowexact_pitch_phi(xt) + (rt + 2) * lowexact_pitch_mu(xt);
+__host__ __device__ constexpr int lowexact_tile_floats(int nx, int ny) {   // one phi tile and its mu tile
+  return (lowexact_rows(ny) + 4) * lowexact_pitch_phi(lowexact_cols(nx)) +
+         (lowexact_rows(ny) + 2) * lowexact_pitch_mu(lowexact_cols(nx));
 }
-__host__ __device__ constexpr int lowexact_smem_floats(int xt, int rt) {
-  return 4 * lowexact_tile_floats(xt, rt) > 2 * kLxValues * kLxWarps * kLxRows ? 4 * lowexact_tile_floats(xt, rt)
+__host__ __device__ constexpr int lowexact_smem_floats(int nx, int ny) {
+  return 2 * lowexact_tile_floats(nx, ny) > 2 * kLxValues * kLxWarps * kLxRows ? 2 * lowexact_tile_floats(nx, ny)
                                                                                 : 2 * kLxValues * kLxWarps * kLxRows;
-}
-// pair arithmetic without renormalising the result (|lo| may reach a few ulps
-// of hi, which the next operation carries)
-__device__ __forceinline__ F2 pair_mul(F2 a, F2 b) {
-  const float p = __fmul_rn(a.hi, b.hi);
-  return F2{p, __fmaf_rn(a.lo, b.hi, __fmaf_rn(a.hi, b.lo, __fmaf_rn(a.hi, b.hi, -p)))};
-}
-__device__ __forceinline__ F2 pair_add(F2 a, F2 b) {
-  const F2 s = two_sum_f(a.hi, b.hi);
-  return F2{s.hi, __fadd_rn(s.lo, __fadd_rn(a.lo, b.lo))};
-}
-__device__ __forceinline__ F2 pair_sub(F2 a, F2 b) {
-  const F2 s = two_sum_f(a.hi, -b.hi);
-  return F2{s.hi, __fadd_rn(s.lo, __fsub_rn(a.lo, b.lo))};
 }
 // acc += F w for an FP32-pair F and a double-float w: the product's rounding
 // error by fused multiply-adds, the low parts added unnormalised
@@ -140,46 +116,43 @@ __device__ __forceinline__ void df_acc_prod(F2& acc, F2 F, float wh, float wl) {
   acc.hi = s.hi;
   acc.lo = __fadd_rn(acc.lo, __fadd_rn(s.lo, e));
 }
-template <int XT>
-__global__ void __launch_bounds__(kLxWarps * 32, 4) k_lowrows_exact(const MemberDesc* __restrict__ descs, int log2nx,
+__global__ void __launch_bounds__(kLxWarps * 32) k_lowrows_exact(const MemberDesc* __restrict__ descs, int log2nx,
                                                                  int log2ny, const float4* __restrict__ twff) {
   const MemberDesc& D = descs[blockIdx.z];
   pdl_wait();
   if (D.low != 2) return;                              // uniform per CTA
   extern __shared__ __align__(16) float sm[];
   const int nx = 1 << log2nx, ny = 1 << log2ny, mx = nx - 1, my = ny - 1;
-  const int RT = lowexact_rows(ny);
-  constexpr int PP = lowexact_pitch_phi(XT), PM = lowexact_pitch_mu(XT);
+  const int XT = lowexact_cols(nx), RT = lowexact_rows(ny);
+  const int PP = lowexact_pitch_phi(XT), PM = lowexact_pitch_mu(XT);
   const int tid = threadIdx.x, nt = blockDim.x;
   const int x0 = blockIdx.x * XT, j0 = blockIdx.y * RT;
   const float* phi = static_cast<const float*>(D.phi);
-  // quarter h = 0..3: phi rows j0 - 2 + r, cols x0 + h nx/4 - 3 + c; mu rows
-  // j0 - 1 + r, cols x0 + h nx/4 - 2 + c
-  const int TF = lowexact_tile_floats(XT, RT);
-#pragma unroll
-  for (int h = 0; h < 4; ++h)
-    for (int e = tid; e < (RT + 4) * (XT + 6); e += nt) {
-      const int r = e / (XT + 6), c = e - r * (XT + 6);
-      sm[h * TF + r * PP + c] =
-          __ldg(phi + ((size_t)((j0 - 2 + r) & my) << log2nx) + ((x0 + h * (nx >> 2) - 3 + c) & mx));
-    }
+  // half h = 0, 1: phi rows j0 - 2 + r, cols x0 + h nx/2 - 3 + c; mu rows
+  // j0 - 1 + r, cols x0 + h nx/2 - 2 + c
+  const int TF = lowexact_tile_floats(nx, ny);
+  for (int e = tid; e < 2 * (RT + 4) * (XT + 6); e += nt) {
+    const int h = e / ((RT + 4) * (XT + 6)), e1 = e - h * (RT + 4) * (XT + 6);
+    const int r = e1 / (XT + 6), c = e1 - r * (XT + 6);
+    sm[h * TF + r * PP + c] =
+        __ldg(phi + ((size_t)((j0 - 2 + r) & my) << log2nx) + ((x0 + h * (nx >> 1) - 3 + c) & mx));
+  }
   __syncthreads();
   const Shear<float> sc(*D.st, true);                  // s^{n+1}
-  {                                                    // mu in FP32, contracted as in the stage-2 stencil
+  {                                                    // mu in FP32, as the stage-2 stencil forms it
     const float a = D.f.a, b = D.f.b, kappa = D.f.kappa;
     const float cxx = 1.f + sc.s * sc.s, cxy = 2.f * sc.s;
     const float kxx = kappa * cxx * D.f.inv_h2, kxy = kappa * cxy * D.f.inv_4h2, kyy = kappa * D.f.inv_h2;
-#pragma unroll
-    for (int h = 0; h < 4; ++h)
-    for (int e = tid; e < (RT + 2) * (XT + 4); e += nt) {
-      const int r = e / (XT + 4), c = e - r * (XT + 4);
-      const float* pc_ = sm + h * TF + (r + 1) * PP + (c + 1);   // the centre in quarter h's phi tile
+    for (int e = tid; e < 2 * (RT + 2) * (XT + 4); e += nt) {
+      const int h = e / ((RT + 2) * (XT + 4)), e1 = e - h * (RT + 2) * (XT + 4);
+      const int r = e1 / (XT + 4), c = e1 - r * (XT + 4);
+      const float* pc_ = sm + h * TF + (r + 1) * PP + (c + 1);   // the centre in half h's phi tile
       const float pc = pc_[0];
       const float sxx = pc_[1] - 2.f * pc + pc_[-1];
       const float syy = pc_[PP] - 2.f * pc + pc_[-PP];
       const float sxy = pc_[PP + 1] - pc_[-PP + 1] - pc_[PP - 1] + pc_[-PP - 1];
-      const float klap = __fmaf_rn(kyy, syy, __fmaf_rn(kxx, sxx, -__fmul_rn(kxy, sxy)));
-      sm[h * TF + (RT + 4) * PP + r * PM + c] = __fmaf_rn(pc, __fmaf_rn(b, __fmul_rn(pc, pc), -a), -klap);
+      const float klap = kxx * sxx - kxy * sxy + kyy * syy;
+      sm[h * TF + (RT + 4) * PP + r * PM + c] = pc * (b * (pc * pc) - a) - klap;
     }
   }
   __syncthreads();
@@ -189,46 +162,35 @@ __global__ void __launch_bounds__(kLxWarps * 32, 4) k_lowrows_exact(const Member
   const int lowm = D.lowm, nv = 2 * (lowm + 1);
   const int tshift = LOG2_NMAX - log2nx;
   const int lane = tid & 31, warp = tid >> 5;
-  constexpr int cw = XT / kLxWarps > 0 ? XT / kLxWarps : 1;      // columns per warp
+  const int cw = XT / kLxWarps > 0 ? XT / kLxWarps : 1;        // columns per warp
   const int c0 = warp * cw, c1 = min(XT, c0 + cw);
   F2 acc[kLxValues];
 #pragma unroll
   for (int k = 0; k < kLxValues; ++k) acc[k] = F2{0.f, 0.f};
-  // 4 h^2 F in double-float at a point, p and q pointing at phi and mu there
+  // F at (row j, col x) of half h in double-float, p and q pointing at phi and mu there
   auto curl = [&](const float* p, const float* q) {
     const F2 dxp = two_sum_f(p[1], -p[-1]);
     const F2 dxm = two_sum_f(q[1], -q[-1]);
-    const F2 dyp = pair_add(pair_mul(W0, two_sum_f(p[PP], -p[-PP])), pair_mul(W1, two_sum_f(p[PP + dd], -p[-PP - dd])));
-    const F2 dym = pair_add(pair_mul(W0, two_sum_f(q[PM], -q[-PM])), pair_mul(W1, two_sum_f(q[PM + dd], -q[-PM - dd])));
-    return pair_sub(pair_mul(dxp, dym), pair_mul(dyp, dxm));
+    const F2 dyp = df_add(df_mul(W0, two_sum_f(p[PP], -p[-PP])), df_mul(W1, two_sum_f(p[PP + dd], -p[-PP - dd])));
+    const F2 dym = df_add(df_mul(W0, two_sum_f(q[PM], -q[-PM])), df_mul(W1, two_sum_f(q[PM + dd], -q[-PM - dd])));
+    return df_mul(df_add(df_mul(dxp, dym), df_neg(df_mul(dyp, dxm))), KF);
   };
   if (lane < RT) {
-    const float* prow = sm + (lane + 2) * PP + 3;                // phi row j, col 0 of quarter 0's tile
+    const float* prow = sm + (lane + 2) * PP + 3;                // phi row j, col 0 of half 0's tile
     const float* mrow = sm + (RT + 4) * PP + (lane + 1) * PM + 2;   // mu row j
-#pragma unroll 1
     for (int c = c0; c < c1; ++c) {
-      const F2 F0 = curl(prow + c, mrow + c), F2_ = curl(prow + 2 * TF + c, mrow + 2 * TF + c);
-      const F2 E0 = pair_add(F0, F2_), O0 = pair_sub(F0, F2_);
-      const F2 F1 = curl(prow + TF + c, mrow + TF + c), F3 = curl(prow + 3 * TF + c, mrow + 3 * TF + c);
-      const F2 E1 = pair_add(F1, F3), O1 = pair_sub(F1, F3);
-      const F2 P = pair_add(E0, E1), M = pair_sub(E0, E1);       // m = 0, 4, 8 and m = 2, 6
-      df_acc(acc[0], P);
+      const F2 Fa = curl(prow + c, mrow + c);                    // x
+      const F2 Fb = curl(prow + TF + c, mrow + TF + c);          // x + nx / 2
+      const F2 E = df_add(Fa, Fb), O = df_add(Fa, df_neg(Fb));   // for even and odd m
+      df_acc(acc[0], E);
       const int x = x0 + c;
 #pragma unroll
       for (int m = 1; m <= kLowMExact; ++m) {
         if (m > lowm) break;
         const float4 w = __ldg(twff + (((m * x) & mx) << tshift));   // cos, sin of 2 pi m x / nx as pairs
-        if (m % 2 == 0) {
-          const F2 G = m % 4 ? M : P;
-          df_acc_prod(acc[2 * m], G, w.x, w.y);
-          df_acc_prod(acc[2 * m + 1], G, -w.z, -w.w);
-        } else {                                       // (O0 + i g O1)(cos - i sin), g = -1 for m = 1, 5
-          const float g = m % 4 == 1 ? -1.f : 1.f;
-          df_acc_prod(acc[2 * m], O0, w.x, w.y);
-          df_acc_prod(acc[2 * m], O1, g * w.z, g * w.w);
-          df_acc_prod(acc[2 * m + 1], O0, -w.z, -w.w);
-          df_acc_prod(acc[2 * m + 1], O1, g * w.x, g * w.y);
-        }
+        const F2 G = (m & 1) ? O : E;
+        df_acc_prod(acc[2 * m], G, w.x, w.y);
+        df_acc_prod(acc[2 * m + 1], G, -w.z, -w.w);
       }
     }
   }
@@ -255,7 +217,6 @@ __global__ void __launch_bounds__(kLxWarps * 32, 4) k_lowrows_exact(const Member
       sum = df_add(sum, F2{red[((2 * v) * kLxWarps + w) * 32 + r], red[((2 * v + 1) * kLxWarps + w) * 32 + r]});
     const int j = j0 + r, m = v >> 1;
     if (nxb == 1) {
-      sum = df_mul(sum, KF);
       reinterpret_cast<float*>(lrh + ((size_t)m << log2ny) + j)[v & 1] = sum.hi;
       reinterpret_cast<float*>(lrl + ((size_t)m << log2ny) + j)[v & 1] = sum.lo;
     } else {
@@ -274,12 +235,10 @@ __global__ void __launch_bounds__(kLxWarps * 32, 4) k_lowrows_exact(const Member
     const int r = e % RT, v = e / RT;
     const int j = j0 + r, m = v >> 1;
     F2 tot{0.f, 0.f};
-#pragma unroll 4
     for (int xb = 0; xb < nxb; ++xb) {
       const float2 pv = __ldcg(part + (((size_t)xb * kLxValues + v) << log2ny) + j);
       tot = df_add(tot, F2{pv.x, pv.y});
     }
-    tot = df_mul(tot, KF);
     reinterpret_cast<float*>(lrh + ((size_t)m << log2ny) + j)[v & 1] = tot.hi;
     reinterpret_cast<float*>(lrl + ((size_t)m << log2ny) + j)[v & 1] = tot.lo;
   }
@@ -287,24 +246,19 @@ __global__ void __launch_bounds__(kLxWarps * 32, 4) k_lowrows_exact(const Member
 }
 
 // ----------------------------------------------------------------- launchers
-static const void* lowexact_fn(int xt) {
-  return xt >= 32 ? (const void*)k_lowrows_exact<32> : xt >= 16 ? (const void*)k_lowrows_exact<16>
-       : xt >= 8  ? (const void*)k_lowrows_exact<8>  : (const void*)k_lowrows_exact<4>;
-}
 void launch_lowrows_exact(const MemberDesc* d, int nmem, int log2nx, int log2ny, const float4* twff,
                           cudaStream_t st) {
   const int nx = 1 << log2nx, ny = 1 << log2ny;
-  const int xt = lowexact_cols(nx, ny);
-  const size_t smem = (size_t)lowexact_smem_floats(xt, lowexact_rows(ny)) * sizeof(float);
-  const dim3 grid((nx / 4) / xt, ny / lowexact_rows(ny), nmem);
+  const size_t smem = (size_t)lowexact_smem_floats(nx, ny) * sizeof(float);
+  const dim3 grid((nx / 2) / lowexact_cols(nx), ny / lowexact_rows(ny), nmem);
   void* args[] = {(void*)&d, (void*)&log2nx, (void*)&log2ny, (void*)&twff};
-  launch_pdl(lowexact_fn(xt), grid, kLxWarps * 32, args, smem, st);
+  launch_pdl((const void*)k_lowrows_exact, grid, kLxWarps * 32, args, smem, st);
 }
 size_t lowrows_bytes(int nx, int ny) {
   // hi and lo planes of the coefficients, the exact path's per-tile sums and
   // its row-block counters
   return 2 * (size_t)(kLowM + 1) * ny * sizeof(float2) +
-         (size_t)((nx / 4) / lowexact_cols(nx, ny)) * kLxValues * ny * sizeof(float2) +
+         (size_t)((nx / 2) / lowexact_cols(nx)) * kLxValues * ny * sizeof(float2) +
          (size_t)(ny / lowexact_rows(ny)) * sizeof(int);
 }
 void launch_step_state_init(const MemberDesc* d, int nmem, cudaStream_t st) {
@@ -334,8 +288,7 @@ void set_step_smem_limits() {
   const int lim = 220 * 1024;   // dynamic part; leaves room for static shared memory
   set_row_smem_limits<T>(lim);
   set_col_smem_limits<T>(lim);
-  if (sizeof(T) == 4)
-    for (int xt : {4, 8, 16, 32}) cudaFuncSetAttribute(lowexact_fn(xt), cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+  if (sizeof(T) == 4) cudaFuncSetAttribute(k_lowrows_exact, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
 }
 
 #define SHF_INST(T)                                                                                      \
