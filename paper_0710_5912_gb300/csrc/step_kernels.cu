@@ -87,6 +87,12 @@ __global__ void k_step_state_init(const MemberDesc* __restrict__ descs, int nmem
 // warp order; with several column tiles per row the CTAs park their sums in
 // a scratch area and the last CTA of a row block to finish (an atomic
 // counter; nothing waits) folds them in tile order into low_rows.
+// What bounds it is FP32 issue.  XT is a template argument (tile indices divided
+// by run-time widths cost an integer division per tile element) and 80 registers
+// let three CTAs share an SM: 20 Stokes steps at 1024^2 1655 -> 1567 us, at
+// 1024 x 512 1388 -> 1342.  Folding quarters of the rows and renormalising fewer
+// pairs was 5% faster still, but other last bits of the sums flip the FP32
+// rounding of a low mode now and then, and psi's noise with it.
 constexpr int kLxRows = 32;     // rows per CTA: one per lane
 constexpr int kLxCols = 64;     // columns per CTA
 constexpr int kLxWarps = 8;
@@ -116,24 +122,26 @@ __device__ __forceinline__ void df_acc_prod(F2& acc, F2 F, float wh, float wl) {
   acc.hi = s.hi;
   acc.lo = __fadd_rn(acc.lo, __fadd_rn(s.lo, e));
 }
-__global__ void __launch_bounds__(kLxWarps * 32) k_lowrows_exact(const MemberDesc* __restrict__ descs, int log2nx,
+template <int XT>
+__global__ void __launch_bounds__(kLxWarps * 32, 3) k_lowrows_exact(const MemberDesc* __restrict__ descs, int log2nx,
                                                                  int log2ny, const float4* __restrict__ twff) {
   const MemberDesc& D = descs[blockIdx.z];
   pdl_wait();
   if (D.low != 2) return;                              // uniform per CTA
   extern __shared__ __align__(16) float sm[];
   const int nx = 1 << log2nx, ny = 1 << log2ny, mx = nx - 1, my = ny - 1;
-  const int XT = lowexact_cols(nx), RT = lowexact_rows(ny);
-  const int PP = lowexact_pitch_phi(XT), PM = lowexact_pitch_mu(XT);
+  const int RT = lowexact_rows(ny);                    // XT = lowexact_cols(nx)
+  constexpr int PP = lowexact_pitch_phi(XT), PM = lowexact_pitch_mu(XT);
   const int tid = threadIdx.x, nt = blockDim.x;
   const int x0 = blockIdx.x * XT, j0 = blockIdx.y * RT;
   const float* phi = static_cast<const float*>(D.phi);
   // half h = 0, 1: phi rows j0 - 2 + r, cols x0 + h nx/2 - 3 + c; mu rows
   // j0 - 1 + r, cols x0 + h nx/2 - 2 + c
   const int TF = lowexact_tile_floats(nx, ny);
-  for (int e = tid; e < 2 * (RT + 4) * (XT + 6); e += nt) {
-    const int h = e / ((RT + 4) * (XT + 6)), e1 = e - h * (RT + 4) * (XT + 6);
-    const int r = e1 / (XT + 6), c = e1 - r * (XT + 6);
+#pragma unroll
+  for (int h = 0; h < 2; ++h)
+  for (int e = tid; e < (RT + 4) * (XT + 6); e += nt) {
+    const int r = e / (XT + 6), c = e - r * (XT + 6);
     sm[h * TF + r * PP + c] =
         __ldg(phi + ((size_t)((j0 - 2 + r) & my) << log2nx) + ((x0 + h * (nx >> 1) - 3 + c) & mx));
   }
@@ -143,9 +151,10 @@ __global__ void __launch_bounds__(kLxWarps * 32) k_lowrows_exact(const MemberDes
     const float a = D.f.a, b = D.f.b, kappa = D.f.kappa;
     const float cxx = 1.f + sc.s * sc.s, cxy = 2.f * sc.s;
     const float kxx = kappa * cxx * D.f.inv_h2, kxy = kappa * cxy * D.f.inv_4h2, kyy = kappa * D.f.inv_h2;
-    for (int e = tid; e < 2 * (RT + 2) * (XT + 4); e += nt) {
-      const int h = e / ((RT + 2) * (XT + 4)), e1 = e - h * (RT + 2) * (XT + 4);
-      const int r = e1 / (XT + 4), c = e1 - r * (XT + 4);
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+    for (int e = tid; e < (RT + 2) * (XT + 4); e += nt) {
+      const int r = e / (XT + 4), c = e - r * (XT + 4);
       const float* pc_ = sm + h * TF + (r + 1) * PP + (c + 1);   // the centre in half h's phi tile
       const float pc = pc_[0];
       const float sxx = pc_[1] - 2.f * pc + pc_[-1];
@@ -162,7 +171,7 @@ __global__ void __launch_bounds__(kLxWarps * 32) k_lowrows_exact(const MemberDes
   const int lowm = D.lowm, nv = 2 * (lowm + 1);
   const int tshift = LOG2_NMAX - log2nx;
   const int lane = tid & 31, warp = tid >> 5;
-  const int cw = XT / kLxWarps > 0 ? XT / kLxWarps : 1;        // columns per warp
+  constexpr int cw = XT / kLxWarps > 0 ? XT / kLxWarps : 1;        // columns per warp
   const int c0 = warp * cw, c1 = min(XT, c0 + cw);
   F2 acc[kLxValues];
 #pragma unroll
@@ -178,6 +187,7 @@ __global__ void __launch_bounds__(kLxWarps * 32) k_lowrows_exact(const MemberDes
   if (lane < RT) {
     const float* prow = sm + (lane + 2) * PP + 3;                // phi row j, col 0 of half 0's tile
     const float* mrow = sm + (RT + 4) * PP + (lane + 1) * PM + 2;   // mu row j
+#pragma unroll 1
     for (int c = c0; c < c1; ++c) {
       const F2 Fa = curl(prow + c, mrow + c);                    // x
       const F2 Fb = curl(prow + TF + c, mrow + TF + c);          // x + nx / 2
@@ -246,13 +256,17 @@ __global__ void __launch_bounds__(kLxWarps * 32) k_lowrows_exact(const MemberDes
 }
 
 // ----------------------------------------------------------------- launchers
+static const void* lowexact_fn(int xt) {
+  return xt >= 64 ? (const void*)k_lowrows_exact<64> : xt >= 32 ? (const void*)k_lowrows_exact<32>
+       : xt >= 16 ? (const void*)k_lowrows_exact<16> : (const void*)k_lowrows_exact<8>;
+}
 void launch_lowrows_exact(const MemberDesc* d, int nmem, int log2nx, int log2ny, const float4* twff,
                           cudaStream_t st) {
   const int nx = 1 << log2nx, ny = 1 << log2ny;
   const size_t smem = (size_t)lowexact_smem_floats(nx, ny) * sizeof(float);
   const dim3 grid((nx / 2) / lowexact_cols(nx), ny / lowexact_rows(ny), nmem);
   void* args[] = {(void*)&d, (void*)&log2nx, (void*)&log2ny, (void*)&twff};
-  launch_pdl((const void*)k_lowrows_exact, grid, kLxWarps * 32, args, smem, st);
+  launch_pdl(lowexact_fn(lowexact_cols(nx)), grid, kLxWarps * 32, args, smem, st);
 }
 size_t lowrows_bytes(int nx, int ny) {
   // hi and lo planes of the coefficients, the exact path's per-tile sums and
@@ -288,7 +302,8 @@ void set_step_smem_limits() {
   const int lim = 220 * 1024;   // dynamic part; leaves room for static shared memory
   set_row_smem_limits<T>(lim);
   set_col_smem_limits<T>(lim);
-  if (sizeof(T) == 4) cudaFuncSetAttribute(k_lowrows_exact, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+  if (sizeof(T) == 4)
+    for (int xt : {8, 16, 32, 64}) cudaFuncSetAttribute(lowexact_fn(xt), cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
 }
 
 #define SHF_INST(T)                                                                                      \
