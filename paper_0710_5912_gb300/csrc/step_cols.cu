@@ -16,7 +16,7 @@ namespace shf {
 // of phi); mode 1: flow (g, omega* -> psi, increment of omega; Stokes: g ->
 // psi).
 template <class T>
-__device__ __forceinline__ void stage_column(cplx<T>* st, const cplx<T>* __restrict__ src, int m, int ny, int t,
+__device__ __forceinline__ void stage_column(cplx<T>* st, const cplx<T>* src, int m, int ny, int t,
                                              int Tc) {
   using C = cplx<T>;
   constexpr int LC = Layout<T>::LC;

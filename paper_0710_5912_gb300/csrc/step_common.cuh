@@ -134,14 +134,6 @@ __device__ __forceinline__ Quad<double> ld4(const double* p) {
   const double2 a = reinterpret_cast<const double2*>(p)[0], b = reinterpret_cast<const double2*>(p)[1];
   return Quad<double>{{a.x, a.y, b.x, b.y}};
 }
-__device__ __forceinline__ Quad<float> ldg4(const float* p) {
-  const float4 a = __ldg(reinterpret_cast<const float4*>(p));
-  return Quad<float>{{a.x, a.y, a.z, a.w}};
-}
-__device__ __forceinline__ Quad<double> ldg4(const double* p) {
-  const double2 a = __ldg(reinterpret_cast<const double2*>(p)), b = __ldg(reinterpret_cast<const double2*>(p) + 1);
-  return Quad<double>{{a.x, a.y, b.x, b.y}};
-}
 __device__ __forceinline__ void st4(float* p, float a, float b, float c, float d) {
   *reinterpret_cast<float4*>(p) = make_float4(a, b, c, d);
 }
@@ -150,13 +142,13 @@ __device__ __forceinline__ void st4(double* p, double a, double b, double c, dou
   reinterpret_cast<double2*>(p)[1] = make_double2(c, d);
 }
 // two reals at an address aligned to two elements
-__device__ __forceinline__ void ldg2(const float* p, float& a, float& b) {
-  const float2 v = __ldg(reinterpret_cast<const float2*>(p));
+__device__ __forceinline__ void ld2(const float* p, float& a, float& b) {
+  const float2 v = *reinterpret_cast<const float2*>(p);
   a = v.x;
   b = v.y;
 }
-__device__ __forceinline__ void ldg2(const double* p, double& a, double& b) {
-  const double2 v = __ldg(reinterpret_cast<const double2*>(p));
+__device__ __forceinline__ void ld2(const double* p, double& a, double& b) {
+  const double2 v = *reinterpret_cast<const double2*>(p);
   a = v.x;
   b = v.y;
 }
@@ -263,6 +255,12 @@ __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wai
 // start earlier (griddepcontrol.launch_dependents): CTAs that arrive while
 // others still run pile up on the SMs with room instead of spreading out, which
 // cost more than the overlap gave (1024^2: 89 us after the wait, 94 at the start).
+// What a step kernel writes (fields, spectra, step state) is read with plain
+// loads, never through the non-coherent path (__ldg, a __restrict__ pointer to
+// const): that path needs memory nothing writes while the kernel lives, and here
+// a kernel lives while its predecessor still writes; nor would the wait order
+// such loads.  Twiddle tables and descriptors, which no step kernel writes, may
+// take it.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
 // launch of a kernel that calls pdl_wait
 inline void launch_pdl(const void* f, dim3 grid, dim3 threads, void** args, size_t smem, cudaStream_t st) {

@@ -138,12 +138,26 @@ __global__ void __launch_bounds__(kLxWarps * 32, 3) k_lowrows_exact(const Member
   // half h = 0, 1: phi rows j0 - 2 + r, cols x0 + h nx/2 - 3 + c; mu rows
   // j0 - 1 + r, cols x0 + h nx/2 - 2 + c
   const int TF = lowexact_tile_floats(nx, ny);
+  // (the loads of four places are in flight before the first store)
+  for (int e0 = tid; e0 < (RT + 4) * (XT + 6); e0 += 4 * nt) {
+    float v[4][2];
 #pragma unroll
-  for (int h = 0; h < 2; ++h)
-  for (int e = tid; e < (RT + 4) * (XT + 6); e += nt) {
-    const int r = e / (XT + 6), c = e - r * (XT + 6);
-    sm[h * TF + r * PP + c] =
-        __ldg(phi + ((size_t)((j0 - 2 + r) & my) << log2nx) + ((x0 + h * (nx >> 1) - 3 + c) & mx));
+    for (int u = 0; u < 4; ++u) {
+      const int e = e0 + u * nt, r = e / (XT + 6), c = e - r * (XT + 6);
+      if (r < RT + 4) {
+        const float* row = phi + ((size_t)((j0 - 2 + r) & my) << log2nx);
+        v[u][0] = row[(x0 - 3 + c) & mx];
+        v[u][1] = row[(x0 + (nx >> 1) - 3 + c) & mx];
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int e = e0 + u * nt, r = e / (XT + 6), c = e - r * (XT + 6);
+      if (r < RT + 4) {
+        sm[r * PP + c] = v[u][0];
+        sm[TF + r * PP + c] = v[u][1];
+      }
+    }
   }
   __syncthreads();
   const Shear<float> sc(*D.st, true);                  // s^{n+1}

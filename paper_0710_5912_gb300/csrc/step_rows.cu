@@ -150,7 +150,7 @@ struct Row12 {
 };
 template <class T>
 __device__ __forceinline__ Row12<T> ld12_row(const T* row, int x0, int mx) {
-  const Quad<T> a = ldg4(row + ((x0 - 4) & mx)), b = ldg4(row + x0), c = ldg4(row + ((x0 + 4) & mx));
+  const Quad<T> a = ld4(row + ((x0 - 4) & mx)), b = ld4(row + x0), c = ld4(row + ((x0 + 4) & mx));
   return Row12<T>{{a.v[0], a.v[1], a.v[2], a.v[3], b.v[0], b.v[1], b.v[2], b.v[3], c.v[0], c.v[1], c.v[2], c.v[3]}};
 }
 // the middle eight (x0 - 2 .. x0 + 5)
@@ -179,7 +179,7 @@ __device__ __forceinline__ Row8<T> mu8(const Row12<T>& U, const Row12<T>& C, con
   return m;
 }
 template <bool NEG, class T>
-__device__ __forceinline__ void stage2_pair(const MemberDesc& D, const T* __restrict__ phi, T* buf, int j0,
+__device__ __forceinline__ void stage2_pair(const MemberDesc& D, const T* phi, T* buf, int j0,
                                             int log2nx, int my, const Shear<T>& sc, int t, int Tf) {
   const int nx = 1 << log2nx, mx = nx - 1;
   const T cxx = T(1) + sc.s * sc.s, cxy = T(2) * sc.s;
@@ -225,7 +225,7 @@ __device__ __forceinline__ void stage2_pair(const MemberDesc& D, const T* __rest
 // of 72, and the windows spilled 436 bytes per thread.  The caller's barrier
 // comes between the two halves.  (Products are spelled out: the two thread
 // groupings must give the same bits.)
-__device__ __forceinline__ void stage2_mu_f64(const MemberDesc& D, const double* __restrict__ phi, double* mu01,
+__device__ __forceinline__ void stage2_mu_f64(const MemberDesc& D, const double* phi, double* mu01,
                                               double* mu23, int j0, int log2nx, int my, const Shear<double>& sc, int t,
                                               int Tf) {
   const int nx = 1 << log2nx, mx = nx - 1;
@@ -236,8 +236,8 @@ __device__ __forceinline__ void stage2_mu_f64(const MemberDesc& D, const double*
     const int x0 = 4 * q;
     auto row6 = [&](int j) {                           // columns x0 - 1 .. x0 + 4
       const double* r = phi + ((size_t)(j & my) << log2nx);
-      const Quad<double> c = ldg4(r + x0);
-      return Six<double>{{__ldg(r + ((x0 - 1) & mx)), c.v[0], c.v[1], c.v[2], c.v[3], __ldg(r + ((x0 + 4) & mx))}};
+      const Quad<double> c = ld4(r + x0);
+      return Six<double>{{r[(x0 - 1) & mx], c.v[0], c.v[1], c.v[2], c.v[3], r[(x0 + 4) & mx]}};
     };
     Six<double> Dn = row6(j0 - 2), C = row6(j0 - 1);
 #pragma unroll
@@ -260,7 +260,7 @@ __device__ __forceinline__ void stage2_mu_f64(const MemberDesc& D, const double*
   }
 }
 template <bool NEG>
-__device__ __forceinline__ void stage2_curl_f64(const MemberDesc& D, const double* __restrict__ phi, const double* mu01,
+__device__ __forceinline__ void stage2_curl_f64(const MemberDesc& D, const double* phi, const double* mu01,
                                                 const double* mu23, double* buf, int j0, int log2nx, int my,
                                                 const Shear<double>& sc, int t, int Tf) {
   const int nx = 1 << log2nx, mx = nx - 1;
@@ -426,9 +426,9 @@ __global__ void __launch_bounds__(rows_max_threads<T>(P, GROUPED), rows_min_ctas
 template <class T>
 __device__ __forceinline__ Row8<T> ld8_row(const T* row, int x0, int mx) {
   T l0, l1, r0, r1;
-  ldg2(row + ((x0 - 2) & mx), l0, l1);
-  const Quad<T> q = ldg4(row + x0);
-  ldg2(row + ((x0 + 4) & mx), r0, r1);
+  ld2(row + ((x0 - 2) & mx), l0, l1);
+  const Quad<T> q = ld4(row + x0);
+  ld2(row + ((x0 + 4) & mx), r0, r1);
   return Row8<T>{{l0, l1, q.v[0], q.v[1], q.v[2], q.v[3], r0, r1}};
 }
 
