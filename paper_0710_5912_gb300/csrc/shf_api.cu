@@ -713,11 +713,15 @@ void enqueue_step(shf_grid* o) {
 // per call).  FP32
 // grids whose fields were set from outside since their last step also get
 // w_hat, omega's 2D transform, recomputed from omega (a row pass and a column
-// pass; members without w_hat skip them).
+// pass; members without w_hat skip them).  What is only recorded into a
+// caller's stream capture may run later, more than once or never: there the
+// state is always formed anew, and nothing counts as done.
 void enqueue_state_init(shf_grid* o) {
-  if (!o->state_valid)
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  const bool recorded = cudaStreamIsCapturing(o->stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone;
+  if (recorded || !o->state_valid)
     for (auto& cl : o->classes) launch_step_state_init(cl.d_desc, (int)cl.members.size(), o->stream);
-  o->state_valid = true;
+  o->state_valid = o->state_valid || !recorded;
   if (o->precision == SHF_FP32 && !o->what_valid) {
     for (auto& cl : o->classes) {
       const int nm = (int)cl.members.size();
@@ -726,8 +730,13 @@ void enqueue_state_init(shf_grid* o) {
       launch_col_kernel<float>(KIND_COLPASS_WINIT, cl.d_desc, nm, cl.log2nx, cl.log2ny,
                                static_cast<const float2*>(o->d_twr), cl.cfg[KIND_COLPASS_FLOW], o->stream);
     }
-    o->what_valid = true;
+    o->what_valid = !recorded;
   }
+}
+// after a failed call: which of its launches ran is not known
+int forget_state(shf_grid* o, int rc) {
+  if (rc != SHF_OK) o->state_valid = o->what_valid = false;
+  return rc;
 }
 
 // k steps.  With several size classes (an ensemble) the classes are
@@ -1023,7 +1032,7 @@ int tune_class(shf_grid* o, SizeClass& cl, Tune* best) {
 // phi_event (a single FP32 grid), the last step is launched directly and
 // phi_event is recorded between its phi passes (after which phi is final) and
 // its flow passes.
-int run_steps(shf_grid* g, long long nsteps, cudaEvent_t phi_event) {
+int enqueue_run(shf_grid* g, long long nsteps, cudaEvent_t phi_event) {
   if (nsteps > 0) enqueue_state_init(g);
   const bool split = phi_event && nsteps > 0;
   long long left = split ? nsteps - 1 : nsteps;
@@ -1057,6 +1066,9 @@ int run_steps(shf_grid* g, long long nsteps, cudaEvent_t phi_event) {
   SHF_CUDA(g, cudaGetLastError());
   g->n += nsteps;
   return SHF_OK;
+}
+int run_steps(shf_grid* g, long long nsteps, cudaEvent_t phi_event) {
+  return forget_state(g, enqueue_run(g, nsteps, phi_event));
 }
 
 }  // namespace
@@ -1423,7 +1435,8 @@ int shf_profile_step(shf_grid* g, int64_t nsteps, double* kernel_ms, int nkinds)
     }
     cudaError_t err = cudaGetLastError();
     if (err == cudaSuccess) err = cudaStreamSynchronize(g->stream);
-    if (err != cudaSuccess) rc = fail(g, SHF_ECUDA, std::string("profiled step: ") + cudaGetErrorString(err));
+    if (err != cudaSuccess)
+      rc = forget_state(g, fail(g, SHF_ECUDA, std::string("profiled step: ") + cudaGetErrorString(err)));
     g->n += nsteps;
   }
   if (rc == SHF_OK) {
@@ -1462,7 +1475,7 @@ int shf_autotune(shf_grid* g, const char* cache_path, int* choices, int nchoices
       t = it->second;
     } else {
       const int rc = g->precision == SHF_FP64 ? tune_class<double>(g, cl, &t) : tune_class<float>(g, cl, &t);
-      if (rc) return fail(g, rc, "autotune: a trial launch failed");
+      if (rc) return forget_state(g, fail(g, rc, "autotune: a trial launch failed"));
       cache[key] = t;
       changed = true;
     }
