@@ -1350,15 +1350,10 @@ int shf_step(shf_grid* g, int64_t nsteps) {
   return run_steps(g, nsteps, nullptr);
 }
 
-int shf_step_host_f32(shf_grid* g, int64_t nsteps, const float* phi_in, const float* psi_in, const float* omega_in,
-                      float* phi_out, float* psi_out, float* omega_out) {
-  if (!g || nsteps < 0) return SHF_EINVAL;
-  if (g->kind != 0) return fail(g, SHF_EINVAL, "shf_step_host_f32 needs a single grid");
-  if (g->precision != SHF_FP32) return fail(g, SHF_EINVAL, "float fields need an FP32 grid");
-  if (!phi_in && (psi_in || omega_in)) return fail(g, SHF_EINVAL, "inputs need phi_in");
+// shf_step_host_f32 behind its checks; after an error copies may be in flight
+static int step_host_run(shf_grid* g, int64_t nsteps, const float* phi_in, const float* psi_in, const float* omega_in,
+                         float* phi_out, float* psi_out, float* omega_out) {
   Member& m = g->members[0];
-  if (!m.params_set) return fail(g, SHF_ESTATE, "shf_set_params must be called before shf_step_host_f32");
-  SHF_CUDA(g, cudaSetDevice(g->device));
   if (!g->io_stream) SHF_CUDA(g, cudaStreamCreateWithFlags(&g->io_stream, cudaStreamNonBlocking));
   if (!g->phi_done) SHF_CUDA(g, cudaEventCreateWithFlags(&g->phi_done, cudaEventDisableTiming));
   if (!g->in_done) SHF_CUDA(g, cudaEventCreateWithFlags(&g->in_done, cudaEventDisableTiming));
@@ -1406,6 +1401,23 @@ int shf_step_host_f32(shf_grid* g, int64_t nsteps, const float* phi_in, const fl
   SHF_CUDA(g, cudaStreamSynchronize(g->stream));
   SHF_CUDA(g, cudaStreamSynchronize(g->io_stream));
   return SHF_OK;
+}
+
+int shf_step_host_f32(shf_grid* g, int64_t nsteps, const float* phi_in, const float* psi_in, const float* omega_in,
+                      float* phi_out, float* psi_out, float* omega_out) {
+  if (!g || nsteps < 0) return SHF_EINVAL;
+  if (g->kind != 0) return fail(g, SHF_EINVAL, "shf_step_host_f32 needs a single grid");
+  if (g->precision != SHF_FP32) return fail(g, SHF_EINVAL, "float fields need an FP32 grid");
+  if (!phi_in && (psi_in || omega_in)) return fail(g, SHF_EINVAL, "inputs need phi_in");
+  if (!g->members[0].params_set) return fail(g, SHF_ESTATE, "shf_set_params must be called before shf_step_host_f32");
+  SHF_CUDA(g, cudaSetDevice(g->device));
+  const int rc = step_host_run(g, nsteps, phi_in, psi_in, omega_in, phi_out, psi_out, omega_out);
+  if (rc != SHF_OK) {                                   // the caller's arrays are its own again on return
+    cudaStreamSynchronize(g->stream);
+    if (g->io_stream) cudaStreamSynchronize(g->io_stream);
+    cudaGetLastError();                                 // reported already
+  }
+  return forget_state(g, rc);
 }
 
 int shf_profile_step(shf_grid* g, int64_t nsteps, double* kernel_ms, int nkinds) {

@@ -40,8 +40,14 @@ int zero_map(void* map) {
 extern "C" {
 const char* fake_log() { return log_.c_str(); }
 void fake_clear() { log_.clear(); }
-void fake_fail_copy(int n) { copies_until_failure = n; }
-void fake_fail_launch(int n) { launches_until_failure = n; }
+void fake_fail_copy(int n) {
+  copies_until_failure = n;
+  last = cudaSuccess;
+}
+void fake_fail_launch(int n) {
+  launches_until_failure = n;
+  last = cudaSuccess;
+}
 void fake_capture(int on) { capturing = on; }
 
 cudaError_t cudaMalloc(void** p, size_t n) { return *p = std::calloc(1, n), cudaSuccess; }

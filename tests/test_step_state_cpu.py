@@ -99,3 +99,17 @@ def test_a_failed_launch_is_not_taken_for_done(run, launch):
     run.step(rc=shf.SHF_ECUDA)
     again = run.step()
     assert has(again, INIT) == 1 and has(again, OMEGA) == 3 and has(again, STAGE1) == 1
+
+
+@pytest.mark.parametrize("copy", range(6))
+def test_no_copy_outlives_a_failed_host_call(run, copy):
+    """Host arrays belong to the caller once the call has returned, and the
+    next call on the grid's stream must not meet this one's uploads."""
+    f = [(ctypes.c_float * (64 * 64))() for _ in range(6)]
+    run.lib.fake_fail_copy(copy)
+    assert run.lib.shf_step_host_f32(run.h, 1, *f) == shf.SHF_ECUDA
+    lines = [line.split() for line in run.log()]
+    for stream in {line[1] for line in lines if line[0] == "copy"}:
+        names = [line[0] for line in lines if line[1] == stream]
+        assert "sync" in names[len(names) - names[::-1].index("copy"):]
+    assert has(run.step(), INIT) == 1
