@@ -374,15 +374,14 @@ MemberDesc make_desc(const shf_grid* o, const Member& m) {
   p.inv_4h2 = 1.0 / (4.0 * m.dx * m.dx);
   p.inv_nxny = 1.0 / ((double)m.nx * (double)m.ny);
   const double two_pi = 6.283185307179586476925286766559;
-  p.qx_unit = two_pi / (m.nx * m.dx);
+  d.qx_unit = two_pi / (m.nx * m.dx);
   p.qy_unit = two_pi / (m.ny * m.dx);
   RealPar<float>& f = d.f;
   f.a = (float)p.a; f.b = (float)p.b; f.kappa = (float)p.kappa; f.dt = (float)p.dt;
   f.c_dt_aM = (float)p.c_dt_aM; f.c_dt_bM = (float)p.c_dt_bM; f.c_hdt_kM = (float)p.c_hdt_kM;
   f.c_hdt_nu = (float)p.c_hdt_nu; f.c_force = (float)p.c_force;
   f.inv_2h = (float)p.inv_2h; f.inv_h2 = (float)p.inv_h2; f.inv_4h2 = (float)p.inv_4h2;
-  f.inv_nxny = (float)p.inv_nxny; f.qx_unit = (float)p.qx_unit; f.qy_unit = (float)p.qy_unit;
-  d.qx_lo = (float)(p.qx_unit - (double)f.qx_unit);
+  f.inv_nxny = (float)p.inv_nxny; f.qy_unit = (float)p.qy_unit;
   const double fs = p.c_force * p.inv_2h * p.inv_2h;
   d.force_scale.x = (float)fs;
   d.force_scale.y = (float)(fs - (double)d.force_scale.x);

@@ -15,8 +15,8 @@ struct StepState {
   long long n;
   long long dK;     // K(n+1) - K(n): nonzero when the strain wraps during the step
   double s0, s1;    // s(t^n), s(t^{n+1})
-  float2 f0, f1;    // s0 and s1 as float pairs (hi, lo): FP32 kernels convert nothing
-  float2 w0, w1;    // Eq. p1y's weights 1 - |s1|/2 and |s1|/2 as float pairs
+  float f0, f1;     // s0 and s1 rounded
+  float2 w0, w1;    // Eq. p1y's weights 1 - |s1|/2 and |s1|/2 as float pairs (hi, lo)
 };
 
 // A member's parameters and derived constants in the working precision.  The
@@ -33,7 +33,7 @@ struct RealPar {
   T c_force;             // -1/rho (inertial) or -1/eta (Stokes), multiplies F
   T inv_2h, inv_h2, inv_4h2;
   T inv_nxny;            // 1 / (nx ny), the inverse-transform normalisation
-  T qx_unit, qy_unit;    // 2 pi / (nx dx), 2 pi / (ny dx)
+  T qy_unit;             // 2 pi / (ny dx)
 };
 
 // Per-member descriptor, resident in device memory (one entry per run of a
@@ -75,7 +75,7 @@ struct MemberDesc {
   double inv_ratio;      // 1 / ratio (exact: a power of two)
   RealPar<double> d;     // parameters and derived constants
   RealPar<float> f;      // the same, rounded
-  float qx_lo;           // qx_unit = f.qx_unit + qx_lo to about 2^-48
+  double qx_unit;        // 2 pi / (nx dx)
   float2 force_scale;    // c_force inv_2h^2 as a float pair (k_lowrows_exact)
   int stokes;            // rho == 0
   int remap;             // 1 when the SHIFT remap is active
@@ -102,6 +102,24 @@ constexpr int kLowN = 16;
 // error twice as large after 200 steps: the rounding at m = 5..8 reaches the
 // lowest modes through the advection of phi
 constexpr int kLowMExact = 8;
+
+// q_x = m q_unit of mode m and the sheared part s q_x of its wavenumber: both
+// products in double, rounded once to the working precision.
+template <class T>
+__host__ __device__ __forceinline__ void sheared_qx(int m, double q_unit, double s, T& qx, T& sqx) {
+  const double q = m * q_unit;
+  qx = (T)q;
+  sqx = (T)(s * q);
+}
+// An FP32 column instance's q_x and s q_x, in shared memory: the instance's
+// first thread forms them in double for all, before the barrier that ends the
+// wait for the item's data.  Five instructions of every thread would hold the
+// SM's FP64 pipe for 16 cycles per warp each; float pairs (about 2^-45) round
+// otherwise than double near a tie, in 15 of 1.8e8 modes.
+struct ModeQ {
+  double q_unit, s;
+  float qx, sqx;
+};
 
 // Strain sawtooth of Section V from the integer step n (same operation order
 // as the host and the oracle; explicit rounding intrinsics keep the compiler

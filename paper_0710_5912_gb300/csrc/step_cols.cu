@@ -32,40 +32,16 @@ __device__ __forceinline__ void stage_column(cplx<T>* st, const cplx<T>* src, in
 template <class T>
 struct ColConsts {
   T norm, qyu, caM, cbM, ckM, cnu, dt;
-  T qxu, qxl, s, sl;                                   // qx_unit and s (FP32: hi and lo parts)
   int ny;
   bool stokes;
-  __device__ __forceinline__ ColConsts(const MemberDesc& D, int mode, int ny_) : ny(ny_), stokes(D.stokes != 0) {
+  __device__ __forceinline__ ColConsts(const MemberDesc& D, int ny_) : ny(ny_), stokes(D.stokes != 0) {
     const RealPar<T>& p = par<T>(D);
     norm = p.inv_nxny; qyu = p.qy_unit; caM = p.c_dt_aM; cbM = p.c_dt_bM; ckM = p.c_hdt_kM; cnu = p.c_hdt_nu;
-    dt = p.dt; qxu = p.qx_unit;
-    const StepState& S = *D.st;                         // s^n for phi, s^{n+1} for flow
-    if constexpr (sizeof(T) == 4) {
-      const float2 sp = mode == 0 ? S.f0 : S.f1;
-      qxl = D.qx_lo; s = sp.x; sl = sp.y;
-    } else {
-      qxl = T(0); s = mode == 0 ? S.s0 : S.s1; sl = T(0);
-    }
-  }
-  // qx = m qx_unit and s qx of mode m, each rounded once to the working
-  // precision: in FP32 both products are float pairs (errors by fused
-  // multiply-adds, about 2^-46), where forming them in double cost every
-  // thread four instructions on the FP64 pipe per item
-  __device__ __forceinline__ void mode_qx(int m, T& qx, T& sqx) const {
-    if constexpr (sizeof(T) == 4) {
-      const float mf = (float)m;
-      const float p = __fmul_rn(mf, qxu);
-      const float e = __fmaf_rn(mf, qxl, __fmaf_rn(mf, qxu, -p));
-      qx = __fadd_rn(p, e);
-      const float ql = __fadd_rn(__fsub_rn(p, qx), e);
-      const float h = __fmul_rn(s, qx);
-      sqx = __fadd_rn(h, __fmaf_rn(sl, qx, __fmaf_rn(s, ql, __fmaf_rn(s, qx, -h))));
-    } else {
-      qx = m * qxu;
-      sqx = s * qx;
-    }
+    dt = p.dt;
   }
 };
+// the strain of a pass: s^n for phi (mode 0), s^{n+1} for the flow
+__device__ __forceinline__ double pass_strain(const MemberDesc& D, int mode) { return mode == 0 ? D.st->s0 : D.st->s1; }
 
 // Quotients of the multipliers: FP32 takes the hardware reciprocal
 // (__fdividef, within 2 ulp; the divisors here lie in [1e-12, 1e3]), FP64 the
@@ -77,7 +53,7 @@ __device__ __forceinline__ double quot(double a, double b) { return a / b; }
 // compile-time pass kind (0: phi; 1: inertial flow; 2: Stokes flow):
 // kind 0: va = phi*_hat -> increment of phi_hat (x norm), vb = f_hat;
 // kinds 1-2: va = g_hat -> psi_hat (x norm), vb = omega*_hat -> increment (x norm).
-// qx and sqx = s q_x as ColConsts::mode_qx forms them.
+// qx and sqx = s q_x as sheared_qx forms them.
 template <int KIND, class T>
 __device__ __forceinline__ void col_multiply_k(const ColConsts<T>& K, int m, T qx, T sqx, int nn, cplx<T>& va,
                                                cplx<T>& vb) {
@@ -248,7 +224,8 @@ __global__ void __launch_bounds__(512, min_ctas<T>()) k_colpass(const MemberDesc
     cp_async_commit();
   };
 
-  const ColConsts<T> K(D, mode, ny);
+  const ColConsts<T> K(D, ny);
+  const double s = pass_strain(D, mode);
 
   const int iters = persistent_iters(nitems, ipc);
   int m = blockIdx.x * ipc + inst;
@@ -270,7 +247,7 @@ __global__ void __launch_bounds__(512, min_ctas<T>()) k_colpass(const MemberDesc
     fft_reg<false>(va, log2ny, t, buf, tws);
     if (two) fft_reg<false>(vb, log2ny, t, buf, tws);
     T qx, sqx;
-    K.mode_qx(mm, qx, sqx);
+    sheared_qx(mm, D.qx_unit, s, qx, sqx);
 #pragma unroll
     for (int q = 0; q < kP; ++q) col_multiply(mode, K, mm, qx, sqx, t + q * Tc, va[q], vb[q]);
     fft_reg<true>(va, log2ny, t, buf, tws);
@@ -418,8 +395,8 @@ __device__ __forceinline__ void colpass_single_body(const MemberDesc& D, int log
   constexpr bool two = KIND == 0 || KIND == 1;          // second input field
   using T = float;
   using C = float2;
-  const int nx = 1 << log2nx, ny = 1 << log2ny;
-  const int Tc = ny / P;
+  constexpr int ny = 1 << log2ny, Tc = ny / P;
+  const int nx = 1 << log2nx;
   const int ipc = blockDim.x / Tc;
   const int inst = threadIdx.x / Tc, t = threadIdx.x - inst * Tc;
   const int nitems = KIND == 4 && !D.wspec ? 0 : nx >> 1;
@@ -433,6 +410,7 @@ __device__ __forceinline__ void colpass_single_body(const MemberDesc& D, int log
   C* what = static_cast<C*>(D.w_hat);
   // a wrap during the step relabels omega_hat^n: (m, n) <- (m, n + m dK)
   C* tws = reinterpret_cast<C*>(smem_raw + (size_t)ipc * colsingle_inst_bytes(ny));
+  __shared__ ModeQ mode_q[256 / Tc];
   stage_tables_to_smem(tws, tw, log2ny, 4, threadIdx.x, blockDim.x);
   pdl_wait();
   const int dK = (KIND == 1 && D.remap) ? (int)(D.st->dK & (ny - 1)) : 0;
@@ -447,12 +425,15 @@ __device__ __forceinline__ void colpass_single_body(const MemberDesc& D, int log
     cp_async_commit();
   };
 
-  const ColConsts<T> K(D, KIND == 0 ? 0 : 1, ny);
+  const ColConsts<T> K(D, ny);
+  if (KIND != 4 && t == 0) mode_q[inst] = ModeQ{D.qx_unit, pass_strain(D, KIND)};
   const int iters = persistent_iters(nitems, ipc);
   int m = blockIdx.x * ipc + inst;
   issue(m);
   for (int it = 0; it < iters; ++it, m += stride) {
     const bool active = m < nitems;
+    const int mm = active ? m : 0;
+    if (KIND != 4 && t == 0) sheared_qx(mm, mode_q[inst].q_unit, mode_q[inst].s, mode_q[inst].qx, mode_q[inst].sqx);
     cp_async_wait_all();
     __syncthreads();
     C a[P], b[P];                                       // the two fields of mode m, rows t + q Tc
@@ -466,7 +447,6 @@ __device__ __forceinline__ void colpass_single_body(const MemberDesc& D, int log
     issue(m + stride);
     fft_reg<false>(a, log2ny, t, buf, tws);
     if (two) fft_reg<false>(b, log2ny, t, buf, tws);
-    const int mm = active ? m : 0;
     if (KIND == 4) {                                    // omega's 2D transform: the new w_hat
       if (active) {
 #pragma unroll
@@ -478,8 +458,7 @@ __device__ __forceinline__ void colpass_single_body(const MemberDesc& D, int log
 #pragma unroll
       for (int q = 0; q < P; ++q) low_override(D, mm, t + q * Tc, ny, a[q]);
     }
-    T qx, sqx;
-    K.mode_qx(mm, qx, sqx);
+    const T qx = mode_q[inst].qx, sqx = mode_q[inst].sqx;
     if (KIND == 1) {
       if (dK) {                                         // stage omega_hat^n so that rows can be relabelled
 #pragma unroll
@@ -567,6 +546,7 @@ __device__ __forceinline__ void colpass_chunk_body(const MemberDesc& D, int log2
   // twiddle table, kColBarBytes of the launch's dynamic shared memory)
   unsigned long long* bar = reinterpret_cast<unsigned long long*>(smem_raw + colchunk_cta_bytes(ny) +
                                                                   stage_table_bytes(log2ny, 4, sizeof(float)));
+  ModeQ* mode_q = reinterpret_cast<ModeQ*>(bar + 2);    // of the CTA's two modes, behind the mbarrier
   unsigned phase = 0;
   if (threadIdx.x == 0) {
     mbar_init(bar, 1);
@@ -586,12 +566,15 @@ __device__ __forceinline__ void colpass_chunk_body(const MemberDesc& D, int log2
     }
   };
 
-  const ColConsts<T> K(D, KIND == 0 ? 0 : 1, ny);
+  const ColConsts<T> K(D, ny);
+  if (KIND != 4 && t == 0) mode_q[sub] = ModeQ{D.qx_unit, pass_strain(D, KIND)};
   const int iters = persistent_iters(nitems, 1);
   int cb = blockIdx.x;
   issue(cb);
   for (int it = 0; it < iters; ++it, cb += stride) {
     const bool active = cb < nitems;
+    const int mm = active ? 2 * cb + sub : sub;
+    if (KIND != 4 && t == 0) sheared_qx(mm, mode_q[sub].q_unit, mode_q[sub].s, mode_q[sub].qx, mode_q[sub].sqx);
     bool ok = true;
     if (active) {
       ok = mbar_wait_bounded(bar, phase);
@@ -618,7 +601,6 @@ __device__ __forceinline__ void colpass_chunk_body(const MemberDesc& D, int log2
     issue(cb + stride);
     fft_reg<false>(a, log2ny, t, buf, tws, sync);
     if (two) fft_reg<false>(b, log2ny, t, buf, tws, sync);
-    const int mm = active ? 2 * cb + sub : sub;
     if (KIND == 4) {                                    // omega's 2D transform: the new w_hat
       store_rows(a, what, cb, active);
       continue;
@@ -627,8 +609,7 @@ __device__ __forceinline__ void colpass_chunk_body(const MemberDesc& D, int log2
 #pragma unroll
       for (int q = 0; q < P; ++q) low_override(D, mm, t + q * Tc, ny, a[q]);
     }
-    T qx, sqx;
-    K.mode_qx(mm, qx, sqx);
+    const T qx = mode_q[sub].qx, sqx = mode_q[sub].sqx;
     if (KIND == 1) {
       if (dK) {                                         // stage omega_hat^n so that rows can be relabelled
 #pragma unroll
@@ -707,9 +688,9 @@ __device__ __forceinline__ void colgroup_body(const MemberDesc& D, const double2
   C v[P];
 #pragma unroll
   for (int q = 0; q < P; ++q) v[q] = in[t + q * Tc];
-  const ColConsts<double> K(D, KIND == 0 ? 0 : 1, ny);
+  const ColConsts<double> K(D, ny);
   double qx, sqx;
-  K.mode_qx(m, qx, sqx);
+  sheared_qx(m, D.qx_unit, pass_strain(D, KIND), qx, sqx);
   fft_reg<false>(v, LN, t, buf, tws, sync);
   if constexpr (two) {
 #pragma unroll

@@ -39,7 +39,7 @@ struct Shear {
   long long dK;   // K(n+1) - K(n): nonzero when the strain wraps during the step
   // next = false: s = s(t^n) (stage 1); next = true: s = s(t^{n+1}) (stages 2-3)
   __device__ __forceinline__ Shear(const StepState& S, bool next) {
-    if constexpr (sizeof(T) == 4) s = next ? S.f1.x : S.f0.x;
+    if constexpr (sizeof(T) == 4) s = next ? S.f1 : S.f0;
     else s = next ? S.s1 : S.s0;
     w1 = (s < T(0) ? -s : s) * T(0.5);
     w0 = T(1) - w1;
@@ -64,8 +64,8 @@ __device__ __forceinline__ void step_state_set(const MemberDesc& D, long long n)
   S->dK = K1 - K0;
   S->s0 = s0;
   S->s1 = s1;
-  S->f0 = float_pair(s0);
-  S->f1 = float_pair(s1);
+  S->f0 = (float)s0;
+  S->f1 = (float)s1;
   S->w0 = float_pair(1.0 - w1);
   S->w1 = float_pair(w1);
 }
