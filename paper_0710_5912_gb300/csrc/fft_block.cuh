@@ -190,11 +190,13 @@ __host__ __device__ constexpr int padded_len(int N) { return N + N / 16; }
 
 // Per-stage twiddle tables.  A stage of radix R = 2^LR after sub-transforms of
 // length Ns = 2^a multiplies input r of butterfly k = j mod Ns by W_L^{k r},
-// L = Ns R.  The table holds, for each (a, LR) with a + LR <= 12, the pair
-// (exp(+2 pi i k / L), exp(+2 pi i 2k / L)) for k = 0..Ns-1 at entries
-// [2 (stage_table_offset(a, LR) + k)], [.. + 1]: one 16-byte load (FP32) per
-// butterfly, and the warp's loads are one contiguous run.  The other factors
-// are products of these two (stage_factors, dit_twiddled).
+// L = Ns R.  For each (a, LR) with a + LR <= 12 the table holds 2 Ns entries
+// from [2 stage_table_offset(a, LR)] on.
+// FP32: the pairs (exp(+2 pi i k / L), exp(+2 pi i 2k / L)), k = 0..Ns-1: one
+// 16-byte load per butterfly, and the warp's loads are one contiguous run; the
+// other factors are products of these two (stage_factors).
+// FP64: exp(+2 pi i j / L), j = 0..2Ns-1, in which dit_twiddled finds all four
+// of its factors, each rounded once.
 __host__ __device__ constexpr int stage_table_offset(int a, int LR) {
   return 4 * ((1 << a) - 1) + (LR - 1) * (1 << a);
 }
@@ -204,7 +206,7 @@ __host__ __device__ constexpr int stage_table_len() { return 2 * 4 * ((1 << 12) 
 // Compact per-length tables in shared memory.  A register transform with
 // 2^LP points per thread multiplies by twiddles only in its stages a = LP,
 // 2 LP, ... (a = log2 Ns < log2 N; the last one of radix 2^(log2 N - a) <=
-// 2^LP).  The compact table holds the Ns pairs of exactly these stages, in
+// 2^LP).  The compact table holds the 2 Ns entries of exactly these stages, in
 // stage order: stage a starts at pair (2^a - 2^LP) / (2^LP - 1), the sum of
 // the earlier stages' 2^b.  Each transform kernel copies it from the global
 // table once per CTA, so the butterflies read their pair from shared memory.
@@ -231,24 +233,12 @@ __device__ __forceinline__ void load_pair(const float2* p, float2& w1, float2& w
   w1 = float2{x.x, x.y};
   w2 = float2{x.z, x.w};
 }
-__device__ __forceinline__ void load_pair(const double2* p, double2& w1, double2& w2) {
-  w1 = p[0];
-  w2 = p[1];
-}
 
 // ---- the arithmetic of the register FFT.  Products whose contraction would
 // depend on their surroundings are spelled out, so that kernels that share a
 // formula give the same bits.
 __device__ __forceinline__ float fma_rn(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 __device__ __forceinline__ double fma_rn(double a, double b, double c) { return __fma_rn(a, b, c); }
-__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
-__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
-template <class C> __device__ __forceinline__ C cmul_rn(C a, C b) {
-  return C{fma_rn(a.x, b.x, -mul_rn(a.y, b.y)), fma_rn(a.x, b.y, mul_rn(a.y, b.x))};
-}
-template <class C> __device__ __forceinline__ C csqr_rn(C a) {
-  return C{fma_rn(a.x, a.x, -mul_rn(a.y, a.y)), mul_rn(a.x + a.x, a.y)};
-}
 
 // -- FP32: radix-R DFTs of additions, the inputs multiplied by W^r first.
 // radix 16 as 4 x 4: radix-4 DFTs over n1 (n = 4 n1 + n2), the factors
@@ -326,13 +316,18 @@ __device__ __forceinline__ void dft_radix(float2* v) {
 //   X[k] = E[k] + (W w_R^k) O[k],  X[k + R/2] = E[k] - (W w_R^k) O[k],
 // so a level of length len has the factors W^{R/len} w_len^k, and each
 // two-point butterfly takes its factor in six fused multiply-adds: four for
-// a + w b and one per component for a - w b = 2a - (a + w b).  10 FP64
+// a + w b and one per component for a - w b = 2a - (a + w b).  9 FP64
 // instructions per point of a radix-8 stage, where separate factors (R - 1
 // products and their powers) and additions took 13; these passes are bound by
-// the FP64 pipe (about 16 cycles of an SM per warp instruction): a 1024^2 step
-// went from 916 to 796 us.  In FP32 the same butterflies gained 3% at 4096^2
-// and nothing below, and re-drew the rounding noise of phi; it keeps the form
-// above.
+// the FP64 pipe (about 16 cycles of an SM per warp instruction).  a - w b carries
+// its partner's rounding as well; the factors come rounded once from the table
+// instead of as products, which more than makes up for it: rms error against
+// 128 bits 1.53e-16 of the result at 64 points and 2.14e-16 at 1024, with
+// separate factors 1.74 and 2.34 (with fused ones from products 1.80 and 2.42).
+// An inertial step of 1024^2: 941 us with separate factors and one stencil per
+// item of stage 2, 745 with factors from products, 732 now.  In FP32 the same butterflies gained 3% at
+// 4096^2 and nothing below, and re-drew the rounding noise of phi; it keeps the
+// form above.
 // (a, b) <- (a + w b, a - w b)
 template <class C> __device__ __forceinline__ void bfly(C& a, C& b, C w) {
   using T = decltype(a.x);
@@ -340,8 +335,13 @@ template <class C> __device__ __forceinline__ void bfly(C& a, C& b, C w) {
   b = C{fma_rn(T(2), a.x, -p.x), fma_rn(T(2), a.y, -p.y)};
   a = p;
 }
-// the same for w = sigma i (a quarter turn) times the given factor: (a, b) <- (a + i s w b, a - i s w b)
-template <bool INV, class C> __device__ __forceinline__ void bfly_quarter(C& a, C& b, C w) { bfly(a, b, mul_si<INV>(w)); }
+// the same with a - w b formed by itself: for the short last stages of radix 2
+// and 4, whose few factors leave the table nothing to make up for
+template <class C> __device__ __forceinline__ void bfly_apart(C& a, C& b, C w) {
+  const C p = C{fma_rn(w.x, b.x, fma_rn(-w.y, b.y, a.x)), fma_rn(w.x, b.y, fma_rn(w.y, b.x, a.y))};
+  b = C{fma_rn(-w.x, b.x, fma_rn(w.y, b.y, a.x)), fma_rn(-w.x, b.y, fma_rn(-w.y, b.x, a.y))};
+  a = p;
+}
 // w = 1, w = sigma i, and w = (1 + sigma i) / sqrt(2) turned by Q quarters
 template <class C> __device__ __forceinline__ void bfly_one(C& a, C& b) { dft2<false>(a, b); }
 template <bool INV, int Q, class C> __device__ __forceinline__ void bfly_eighth(C& a, C& b) {
@@ -358,7 +358,6 @@ template <int LR> __host__ __device__ constexpr int bit_reversed(int r) {
   for (int i = 0; i < LR; ++i) v |= ((r >> i) & 1) << (LR - 1 - i);
   return v;
 }
-constexpr double kCos8 = 0.70710678118654752440084436210484903928;
 // y holds the R inputs in bit-reversed places, factors all one; X in natural order
 template <bool INV, int LR, class C>
 __device__ __forceinline__ void dit_plain(C* y) {
@@ -384,33 +383,39 @@ __device__ __forceinline__ void dit_plain(C* y) {
       bfly_eighth<INV, 1>(y[i + 3], y[i + 7]);
     }
 }
-// the same with the factors W^r, w1 = W and w2 = W^2 given (already of the transform's sign)
+// the same with the factors W^r, W = W_L^k: w1 = W, w2 = W^2, w4 = W^4 and w1
+// turned by an eighth are entries k, 2k, 4k (a quarter turn on from 2 Ns) and
+// k + Ns of the stage's table
 template <bool INV, int LR, class C>
-__device__ __forceinline__ void dit_twiddled(C* y, C w1, C w2) {
-  using T = decltype(y[0].x);
+__device__ __forceinline__ void dit_twiddled(C* y, const C* tab, int Ns, int k) {
   constexpr int R = 1 << LR;
-  const T sg = INV ? T(1) : T(-1);
-  const C w4 = LR >= 3 ? csqr_rn(w2) : w2;
-  const C e8 = C{T(kCos8), sg * T(kCos8)};
+  auto factor = [&](int j) { return INV ? tab[j] : cconj(tab[j]); };
+  if constexpr (LR == 3) {
+    C w4 = factor((4 * k) & (2 * Ns - 1));
+    if (4 * k >= 2 * Ns) w4 = mul_si<INV>(w4);
 #pragma unroll
-  for (int i = 0; i < R; i += 2) bfly(y[i], y[i + 1], LR == 3 ? w4 : LR == 2 ? w2 : w1);
-  if (LR >= 2) {
-    const C w = LR == 3 ? w2 : w1;
+    for (int i = 0; i < R; i += 2) bfly(y[i], y[i + 1], w4);
+    const C w2 = factor(2 * k);
 #pragma unroll
     for (int i = 0; i < R; i += 4) {
-      bfly(y[i], y[i + 2], w);
-      bfly_quarter<INV>(y[i + 1], y[i + 3], w);
+      bfly(y[i], y[i + 2], w2);
+      bfly(y[i + 1], y[i + 3], mul_si<INV>(w2));
     }
-  }
-  if (LR >= 3) {
-    const C we = cmul_rn(w1, e8);
-#pragma unroll
-    for (int i = 0; i < R; i += 8) {
-      bfly(y[i], y[i + 4], w1);
-      bfly(y[i + 1], y[i + 5], we);
-      bfly_quarter<INV>(y[i + 2], y[i + 6], w1);
-      bfly_quarter<INV>(y[i + 3], y[i + 7], we);
+    const C w1 = factor(k);
+    bfly(y[0], y[4], w1);
+    bfly(y[2], y[6], mul_si<INV>(w1));
+    const C we = factor(k + Ns);
+    bfly(y[1], y[5], we);
+    bfly(y[3], y[7], mul_si<INV>(we));
+  } else {
+    if constexpr (LR == 2) {
+      const C w2 = factor(2 * k);
+      bfly_apart(y[0], y[1], w2);
+      bfly_apart(y[2], y[3], w2);
     }
+    const C w1 = factor(k);
+    bfly_apart(y[0], y[R / 2], w1);
+    if constexpr (LR == 2) bfly_apart(y[1], y[3], mul_si<INV>(w1));
   }
 }
 
@@ -451,18 +456,18 @@ __device__ __forceinline__ void fft_reg_stage(C (&v)[P], int log2N, int log2Ns, 
     const int k = j & (Ns - 1);
 #pragma unroll
     for (int r = 0; r < R; ++r) w[sizeof(w[0].x) == 4 ? r : bit_reversed<LR>(r)] = v[b + r * B];
-    C w1, w2;
-    if (log2Ns > 0) load_pair(twt + 2 * (compact_stage_offset(log2Ns, log2_points<P>()) + k), w1, w2);
+    const C* tab = twt + 2 * compact_stage_offset(log2Ns, log2_points<P>());
     if constexpr (sizeof(w[0].x) == 4) {
       if (log2Ns > 0) {
-        C f[R];
+        C w1, w2, f[R];
+        load_pair(tab + 2 * k, w1, w2);
         stage_factors<R>(w1, w2, f);
 #pragma unroll
         for (int r = 1; r < R; ++r) w[r] = cmul(w[r], INV ? f[r] : cconj(f[r]));
       }
       dft_radix<INV, LR>(w);
     } else {
-      if (log2Ns > 0) dit_twiddled<INV, LR>(w, INV ? w1 : cconj(w1), INV ? w2 : cconj(w2));
+      if (log2Ns > 0) dit_twiddled<INV, LR>(w, tab, Ns, k);
       else dit_plain<INV, LR>(w);
     }
     if (LAST) {
