@@ -197,8 +197,9 @@ int shf_gradient_tensor(shf_grid* g, double G[3], double lengths[2]);
  * that write scratch buffers run, so the state (fields, step) is unchanged and
  * results stay within the parity tolerances (the variants round differently).
  * cache_path (nullable): a JSON file of earlier choices keyed by
- * "NXxNY:fp32|fp64:inertial|stokes|mixed"; keys found there are applied
- * without trials, new ones are added.  choices (nullable, nchoices ints):
+ * "NXxNY:fp32|fp64:inertial|stokes|mixed", with ":N" for a class of N > 1
+ * members; keys found there are applied without trials, new ones are added.
+ * Entries timed with other launch rules ("launch") are timed again.  choices (nullable, nchoices ints):
  * receives (stage1_points, stage2_points) per size class,
  * in order of first appearance among the members.  Parameters must be set.  Not for member
  * views.  SHF_EIO if the cache cannot be written.  The paper has no

@@ -932,17 +932,24 @@ int sf_sums(shf_grid* g, double* S_binned, int nbins, double sums[kSfMoments]) {
 // ------------------------------------------------------------- autotuning
 namespace {
 
+// The number of members is part of the key: thread groups (stage_groups) are
+// taken with 16 points only and while all members' row pairs fit on the chip, so
+// what is faster for many members need not be for one.
 std::string tune_key(const shf_grid* o, const SizeClass& cl) {
   bool inertial = false, stokes = false;
   for (int r : cl.members) (o->members[r].rho > 0 ? inertial : stokes) = true;
   char buf[96];
-  std::snprintf(buf, sizeof(buf), "%dx%d:%s:%s", cl.nx, cl.ny, o->precision == SHF_FP64 ? "fp64" : "fp32",
-                inertial && stokes ? "mixed" : (inertial ? "inertial" : "stokes"));
+  int n = std::snprintf(buf, sizeof(buf), "%dx%d:%s:%s", cl.nx, cl.ny, o->precision == SHF_FP64 ? "fp64" : "fp32",
+                        inertial && stokes ? "mixed" : (inertial ? "inertial" : "stokes"));
+  if (cl.members.size() > 1) std::snprintf(buf + n, sizeof(buf) - n, ":%zu", cl.members.size());
   return buf;
 }
 
 // cache file: a JSON object, one entry per line:
-//   "NXxNY:fp32:inertial": {"stage1_points": 16, "stage2_points": 16},
+//   "NXxNY:fp32:inertial": {"stage1_points": 16, "stage2_points": 16, "launch": 2},
+// "launch" numbers the rules of the launch shapes that the entry was timed with;
+// entries of other rules (the first had no number) are timed again.
+constexpr int kTuneLaunch = 2;
 std::map<std::string, Tune> read_tune_cache(const char* path) {
   std::map<std::string, Tune> m;
   if (!path) return m;
@@ -952,8 +959,10 @@ std::map<std::string, Tune> read_tune_cache(const char* path) {
   while (std::fgets(line, sizeof(line), f)) {
     char key[256];
     Tune t;
-    if (std::sscanf(line, " \"%255[^\"]\": {\"stage1_points\": %d, \"stage2_points\": %d", key, &t.stage1_points,
-                    &t.stage2_points) == 3)
+    int launch = 0;
+    if (std::sscanf(line, " \"%255[^\"]\": {\"stage1_points\": %d, \"stage2_points\": %d, \"launch\": %d", key,
+                    &t.stage1_points, &t.stage2_points, &launch) == 4 &&
+        launch == kTuneLaunch && (t.stage1_points == 8 || t.stage1_points == 16))
       m[key] = t;
   }
   std::fclose(f);
@@ -966,8 +975,8 @@ bool write_tune_cache(const char* path, const std::map<std::string, Tune>& m) {
   std::fprintf(f, "{\n");
   size_t i = 0;
   for (const auto& kv : m) {
-    std::fprintf(f, "  \"%s\": {\"stage1_points\": %d, \"stage2_points\": %d}%s\n", kv.first.c_str(),
-                 kv.second.stage1_points, kv.second.stage2_points, ++i < m.size() ? "," : "");
+    std::fprintf(f, "  \"%s\": {\"stage1_points\": %d, \"stage2_points\": %d, \"launch\": %d}%s\n", kv.first.c_str(),
+                 kv.second.stage1_points, kv.second.stage2_points, kTuneLaunch, ++i < m.size() ? "," : "");
   }
   std::fprintf(f, "}\n");
   return std::fclose(f) == 0;

@@ -1,4 +1,4 @@
-"""What the host keeps about the device's step state between calls, on a fake
+"""What the host keeps between calls (step state, tuned choices), on a fake
 CUDA runtime (fake_cudart.cpp) that logs copies and launches: a call that was
 only captured into the caller's graph, or whose launches failed, has left
 nothing that a later call may rely on."""
@@ -113,3 +113,36 @@ def test_no_copy_outlives_a_failed_host_call(run, copy):
         names = [line[0] for line in lines if line[1] == stream]
         assert "sync" in names[len(names) - names[::-1].index("copy"):]
     assert has(run.step(), INIT) == 1
+
+
+def tune(run, path):
+    out = (ctypes.c_int * 2)()
+    assert run.lib.shf_autotune(run.h, str(path).encode(), out, 2) == 0
+    return out[0], has(run.log(), STAGE1)               # the choice and the trial launches
+
+
+def test_tuned_choices_are_taken_from_like_runs_only(run, tmp_path):
+    """On this runtime every launch takes the same time, and 8 points are tried
+    first: a trial ends with 8, a cached 16 is seen to be applied."""
+    path = tmp_path / "tune.json"
+    old = '"64x64:fp32:inertial": {"stage1_points": 16, "stage2_points": 16'
+    path.write_text("{\n  %s, \"launch\": 2}\n}\n" % old)
+    assert tune(run, path) == (16, 0)
+    for line in (old + "}",                             # timed before thread groups
+                 old.replace("16, ", "7, ") + ', "launch": 2}',     # no variant
+                 old.replace('inertial"', 'inertial:96"') + ', "launch": 2}'):
+        path.write_text("{\n  %s\n}\n" % line)
+        choice, trials = tune(run, path)
+        assert choice == 8 and trials > 0
+        assert '"64x64:fp32:inertial": {"stage1_points": 8, ' in path.read_text()
+
+
+def test_tuned_choices_of_many_members_have_their_own_entry(fake, tmp_path):
+    path, n = tmp_path / "tune.json", 5
+    ens, sizes = ctypes.c_void_p(), (ctypes.c_int * n)(*[64] * n)
+    params = (ctypes.c_double * (8 * n))(*[1.0, 1.0, 1.0, 1.0, 1.0, 1.0, 0.1, 0.01] * n)
+    assert fake.shf_create_ensemble(ctypes.byref(ens), n, sizes, sizes, None, params, None, 0.0, shf.SHF_FP32, None) == 0
+    assert fake.shf_autotune(ens, str(path).encode(), None, 0) == 0
+    assert '"64x64:fp32:inertial:5"' in path.read_text()
+    fake.shf_destroy_grid(ens)
+    fake.fake_clear()
