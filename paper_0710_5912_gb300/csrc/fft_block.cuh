@@ -361,9 +361,7 @@ template <int LR> __host__ __device__ constexpr int bit_reversed(int r) {
 // y holds the R inputs in bit-reversed places, factors all one; X in natural order
 template <bool INV, int LR, class C>
 __device__ __forceinline__ void dit_plain(C* y) {
-  using T = decltype(y[0].x);
   constexpr int R = 1 << LR;
-  const T sg = INV ? T(1) : T(-1);
 #pragma unroll
   for (int i = 0; i < R; i += 2) bfly_one(y[i], y[i + 1]);
   if (LR >= 2)

@@ -43,62 +43,42 @@ struct ColConsts {
 // the strain of a pass: s^n for phi (mode 0), s^{n+1} for the flow
 __device__ __forceinline__ double pass_strain(const MemberDesc& D, int mode) { return mode == 0 ? D.st->s0 : D.st->s1; }
 
-// Quotients of the multipliers: FP32 takes the hardware reciprocal
-// (__fdividef, within 2 ulp; the divisors here lie in [1e-12, 1e3]), FP64 the
-// IEEE quotient.
+// Quotients of the FP32 multipliers: the hardware reciprocal (__fdividef, within
+// 2 ulp; the divisors here lie in [1e-12, 1e3]).
 __device__ __forceinline__ float quot(float a, float b) { return __fdividef(a, b); }
-__device__ __forceinline__ double quot(double a, double b) { return a / b; }
 
-// The multiplier at mode (m, row nn) of the column transform, in place, for a
-// compile-time pass kind (0: phi; 1: inertial flow; 2: Stokes flow):
-// kind 0: va = phi*_hat -> increment of phi_hat (x norm), vb = f_hat;
-// kinds 1-2: va = g_hat -> psi_hat (x norm), vb = omega*_hat -> increment (x norm).
-// qx and sqx = s q_x as sheared_qx forms them.
-template <int KIND, class T>
-__device__ __forceinline__ void col_multiply_k(const ColConsts<T>& K, int m, T qx, T sqx, int nn, cplx<T>& va,
-                                               cplx<T>& vb) {
-  using C = cplx<T>;
+// The FP32 multiplier at mode (m, row nn) of the column transform, in place, for
+// the phi pass (KIND 0: va = phi*_hat -> increment of phi_hat (x norm), vb =
+// f_hat) and the Stokes flow (KIND 2: va = g_hat -> psi_hat (x norm)); inertial
+// members: col_multiply_wspec.  qx and sqx = s q_x as sheared_qx forms them.
+template <int KIND>
+__device__ __forceinline__ void col_multiply_k(const ColConsts<float>& K, int m, float qx, float sqx, int nn, float2& va,
+                                               float2& vb) {
   const int ns = nn < (K.ny >> 1) ? nn : nn - K.ny;
-  const T ky = (T)ns * K.qyu - sqx;
-  const T k2 = qx * qx + ky * ky;
+  const float ky = (float)ns * K.qyu - sqx;
+  const float k2 = qx * qx + ky * ky;
   const bool nyq_row = nn == (K.ny >> 1);
-  const T norm = K.norm;
+  const float norm = K.norm;
   if (KIND == 0) {
-    const C P = va, F = vb;
+    const float2 P = va, F = vb;
     if (nyq_row) {
-      va = C{-P.x * norm, -P.y * norm};                 // Nyquist row of phi^{n+1} -> 0
+      va = float2{-P.x * norm, -P.y * norm};            // Nyquist row of phi^{n+1} -> 0
     } else {
-      const T c4 = K.ckM * (k2 * k2);
-      const T aa = K.caM * k2 - T(2) * c4;
-      const T bbm = K.cbM * k2;
-      const T inv = quot(norm, T(1) + c4);
-      va = C{(aa * P.x - bbm * F.x) * inv, (aa * P.y - bbm * F.y) * inv};
+      const float c4 = K.ckM * (k2 * k2);
+      const float aa = K.caM * k2 - 2.f * c4;
+      const float bbm = K.cbM * k2;
+      const float inv = quot(norm, 1.f + c4);
+      va = float2{(aa * P.x - bbm * F.x) * inv, (aa * P.y - bbm * F.y) * inv};
     }
   } else {
-    const bool zero = nyq_row || (m == 0 && nn == 0);
-    const C G = va;
-    if (KIND == 2) {
-      const T inv = zero ? T(0) : quot(norm, k2 * k2);
-      va = C{G.x * inv, G.y * inv};
-    } else {
-      const C Wv = vb;
-      if (zero) {
-        va = C{T(0), T(0)};
-        vb = C{-Wv.x * norm, -Wv.y * norm};             // omega^{n+1} -> 0 there
-      } else {
-        const T cc = K.cnu * k2;
-        const T inv = quot(T(1), T(1) + cc);
-        const C dw = C{(-T(2) * cc * Wv.x + K.dt * G.x) * inv, (-T(2) * cc * Wv.y + K.dt * G.y) * inv};
-        const T ik = quot(norm, k2);
-        va = C{(Wv.x + dw.x) * ik, (Wv.y + dw.y) * ik};
-        vb = C{dw.x * norm, dw.y * norm};
-      }
-    }
+    const float inv = nyq_row || (m == 0 && nn == 0) ? 0.f : quot(norm, k2 * k2);
+    va = float2{va.x * inv, va.y * inv};
   }
 }
-// The same for FP64 with every operation spelled out: k_colpass and k_colgroup
-// share it and must give the same bits, and the compiler contracts products by
-// their surroundings.
+// The FP64 multiplier (kind 0 and 2 as above; kind 1, inertial flow: va = g_hat ->
+// psi_hat (x norm), vb = omega*_hat -> increment (x norm)) with every operation
+// spelled out: k_colpass and k_colgroup share it and must give the same bits, and
+// the compiler contracts products by their surroundings.
 template <int KIND>
 __device__ __forceinline__ void col_multiply_d(const ColConsts<double>& K, int m, double qx, double sqx, int nn,
                                                double2& va, double2& vb) {
