@@ -298,8 +298,9 @@ __global__ void __launch_bounds__(512) k_sf_rows(const T* __restrict__ f, cplx<T
 // Partials per CTA (kSfMoments): sum S, sum k S, sum S/k, and for the tensor
 // of Eq. L_matrix sum q_cx^2 S, sum q_cx q_cy S, sum q_cy^2 S, sum S with
 // k = 0 included.
-// What bounds it is the FP64 pipe (16 cycles of an SM per warp instruction).
-// Every addition is compensated.  A thread's eight modes lie in one column, so
+// What bounds it is FP64 work (16 cycles of an SM per warp instruction): at
+// 1024^2, 128 CTAs, the pipe of an SM that has one is 55% busy, the rest is the
+// latency of its chains.  Every addition is compensated.  A thread's eight modes lie in one column, so
 // q_x leaves their sums, and the threads' sums meet in shared memory, one warp
 // per moment (a tree of shuffles adds every lane's six pairs at each level).
 // For the bins: along a column k grows

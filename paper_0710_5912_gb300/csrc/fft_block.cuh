@@ -7,7 +7,7 @@
 // their auto-sorted positions, so the output comes out in natural order with no
 // bit reversal.
 //
-// - fft_reg (the step kernels): each thread holds P = 8 (or 16)
+// - fft_reg (the step kernels): each thread holds P = 8 (FP64) or 16 (FP32)
 //   complex values in registers; a stage is radix P (one butterfly per
 //   thread), or radix 8 / 4 / 2 for the last stage; stages exchange through a
 //   padded shared buffer.  Twiddles come from per-stage tables (below), copied
@@ -167,7 +167,7 @@ __device__ void fft_smem(C* const (&buf)[NB], int log2N, int tid, const C* __res
 }
 
 // ---------------------------------------------------------------------------
-// Register-resident FFT (P = 8 points per thread).
+// Register-resident FFT (P = 8 or 16 points per thread).
 //
 // Thread t of an instance (0 <= t < T = N/P) holds v[q] = x[t + T q],
 // q = 0..P-1.  Each Stockham stage is radix P except possibly the last (radix
@@ -178,9 +178,9 @@ __device__ void fft_smem(C* const (&buf)[NB], int log2N, int tid, const C* __res
 // transform ends in registers with v[q] = X[t + T q].  Only the stages in
 // between exchange through shared memory.  Exchange buffers are padded by one
 // element per 16 (index i -> i + i/16), which keeps the scatter of the early
-// stages free of bank conflicts.  The column passes use eight points per
-// thread (P = 16 with one mode per instance measured no faster there); the
-// FP32 row passes use sixteen, one exchange fewer, which measured faster.
+// stages free of bank conflicts.  FP32 uses sixteen points per thread, one
+// exchange fewer, which measured faster; FP64, with twice the registers per
+// point, eight.
 constexpr int kP = 8;
 constexpr int kLogP = 3;
 

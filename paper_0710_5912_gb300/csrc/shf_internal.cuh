@@ -174,18 +174,17 @@ __host__ __device__ constexpr size_t rowinv_inst_bytes(int nx, size_t real_bytes
   return round128(((size_t)nx + (size_t)padded_len(nx)) * 2 * real_bytes);
 }
 // the compact twiddle table that follows the instances of a transform kernel
-// (2^LP points per thread): two complex values per pair
+// (2^LP points per thread): two complex values per butterfly
 __host__ __device__ constexpr size_t stage_table_bytes(int log2n, int LP, size_t real_bytes) {
   return round128((size_t)compact_stage_pairs(log2n, LP) * 4 * real_bytes);
 }
 
-// Row transforms come in two variants, P = 8 points per thread (radix-8
-// stages, 512-thread CTAs) and P = 16 (radix-16 stages, 256-thread CTAs, FP32
-// only); the column passes use 8 points and 512 threads.  The fused stage-1
-// pass's P and the stage-2 stencil tile height are tuning knobs
-// (shf_autotune); the FP32 g row pass uses P = 16 (its first radix-16 stage
-// yields the force's low modes) and the FP32 inverse rows P = 16 (8% faster
-// than 8 in the flow pass, equal in the phi pass at 4096^2).
+// Row transforms hold P = 8 points per thread (radix-8 stages, 512-thread CTAs;
+// FP64) or P = 16 (radix-16 stages, 256-thread CTAs; FP32).  P of the FP32
+// stage-1 pass is a tuning knob (shf_autotune); the FP32 g row pass needs P = 16
+// (its first radix-16 stage yields the force's low modes), and the FP32 inverse
+// rows are 8% faster with 16 in the flow pass at 4096^2, equal in the phi pass.
+// The column passes hold 8 points in FP64 and 16 in FP32.
 constexpr int rowfwd_cta_threads(int P) { return P == 16 ? 256 : 512; }
 // launch bounds of the forward row passes: with P = 16 three CTAs of one group
 // or up to three groups of 256 threads in one CTA (stage_groups); with P = 8

@@ -87,12 +87,16 @@ __global__ void k_step_state_init(const MemberDesc* __restrict__ descs, int nmem
 // warp order; with several column tiles per row the CTAs park their sums in
 // a scratch area and the last CTA of a row block to finish (an atomic
 // counter; nothing waits) folds them in tile order into low_rows.
-// What bounds it is FP32 issue.  XT is a template argument (tile indices divided
-// by run-time widths cost an integer division per tile element) and 80 registers
-// let three CTAs share an SM: 20 Stokes steps at 1024^2 1655 -> 1567 us, at
-// 1024 x 512 1388 -> 1342.  Folding quarters of the rows and renormalising fewer
-// pairs was 5% faster still, but other last bits of the sums flip the FP32
-// rounding of a low mode now and then, and psi's noise with it.
+// What bounds it at 1024^2 (256 CTAs, one or two per SM of 152; 30 us) and 1024 x
+// 512 (128 CTAs; 28 us) is latency: 48 and 29% of the issue slots of the busy
+// schedulers, the rest mostly waiting for the twiddles' loads.  From 2048^2 on
+// (1024 CTAs) the 80 registers let three CTAs share an SM.  XT is a template
+// argument (tile indices divided by run-time widths cost an integer division per
+// tile element): 20 Stokes steps at 1024^2 1655 -> 1567 us, at 1024 x 512 1388 ->
+// 1342; and 1553 and 1320 with four places of a tile loaded before the first
+// store.  Folding quarters of the rows and renormalising fewer pairs was 5%
+// faster still, but other last bits of the sums flip the FP32 rounding of a low
+// mode now and then, and psi's noise with it.
 constexpr int kLxRows = 32;     // rows per CTA: one per lane
 constexpr int kLxCols = 64;     // columns per CTA
 constexpr int kLxWarps = 8;

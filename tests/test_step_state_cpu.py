@@ -21,7 +21,7 @@ INIT, OMEGA, STAGE1 = "k_step_state_init", "k_colpass_single", "k_stage1_rows"
 def fake(tmp_path_factory):
     if shutil.which("g++") is None:
         pytest.skip("no host compiler")
-    _native.build()
+    _native.build(force=not glob.glob(os.path.join(_native.BUILD_DIR, "*.o")))
     out = str(tmp_path_factory.mktemp("fake") / "libshf_fake.so")
     cuda = os.path.join(os.path.dirname(os.path.dirname(_native.nvcc_path())), "include")
     subprocess.run(["g++", "-std=c++17", "-shared", "-fPIC", "-Wl,-Bsymbolic", "-I", cuda, "-o", out,
